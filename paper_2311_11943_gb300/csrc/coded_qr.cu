@@ -27,7 +27,7 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-  size_t Q, R, Gt, Gh, Gt_t, Gh_t, Kpo, part, bar, status, P, Rb, Pt, yw, xw, plans, cg, tc, total;
+  size_t Q, R, Gt, Gh, Gt_t, Gh_t, Kpo, part, blk, bar, status, P, Rb, Pt, yw, xw, plans, cg, tc, total;
 };
 
 struct Buffers {
@@ -39,6 +39,7 @@ struct Buffers {
   void* Gh_t;
   void* Kpo;  // (I_f + G~ G~^T)^{-1}: f x f doubles, then f x f in the storage type
   void* part;
+  void* blk;  // sub-block panel: tag count, sums and partial sums
   unsigned* bar;
   int* status;
   void* P;
@@ -128,6 +129,7 @@ Layout make_layout(const cqr_config* c, const Geo& g, int num_sms) {
   L.Gh_t = take((size_t)(g.f * c->p_c + 1) * s);
   L.Kpo = take((size_t)kMaxF * kMaxF * (8 + s));
   L.part = take(panel_partial_bytes(bmax, s, num_sms));
+  L.blk = take(panel_blk_bytes(bmax, s, num_sms));
   L.bar = take(256);
   L.status = take(256);
   L.P = take((size_t)kMaxSplits * bmax * g.N * s);
@@ -188,6 +190,8 @@ struct cqr_handle_s {
   PanelPlan plan{};
   int plan_bk = -1;
   bool reg_ok = false;
+  bool blk_ok = false;  // the sub-block panel fits
+  PanelBlkPlan blk{};
   // sub-panel schedule of panels too tall for one cluster (FP32): width and cluster plan
   int sub_bs = 0;
   PanelPlan sub_plan{};
@@ -274,6 +278,7 @@ cqr_status setup(cqr_handle h) {
   h->B.Gh_t = base + L.Gh_t;
   h->B.Kpo = base + L.Kpo;
   h->B.part = base + L.part;
+  h->B.blk = base + L.blk;
   h->B.bar = reinterpret_cast<unsigned*>(base + L.bar);
   h->B.status = reinterpret_cast<int*>(base + L.status);
   h->B.P = base + L.P;
@@ -372,10 +377,21 @@ int choose_splits(int bk, int64_t w, int64_t K, int num_sms) {
   return s;
 }
 
+// Whether a comparison switch asks for one of the per-column panel kernels.
+bool column_panel_requested() {
+  auto is = [](const char* name, char v) { const char* e = getenv(name); return e && e[0] == v; };
+  const char* rpl = getenv("CQR_PANEL_RPL");
+  return is("CQR_PANEL_REG", '0') || is("CQR_PANEL_CLUSTER", '0') || is("CQR_PANEL_HIER", '0') ||
+         is("CQR_PANEL_SUB", '1') || (rpl && atoi(rpl) > 0);
+}
+
 template <typename T>
 void ensure_panel_plan(cqr_handle h, int bk) {
   if (bk == h->plan_bk) return;
   const Geo& g = h->g;
+  const bool icgs_or_mgs = h->cfg.panel == CQR_PANEL_ICGS || h->cfg.panel == CQR_PANEL_MGS;
+  h->blk_ok = icgs_or_mgs && !column_panel_requested() &&
+              plan_panel_blk(g.M, bk, sizeof(T), h->num_sms, &h->blk);
   h->plan = plan_panel(g.M, bk, sizeof(T), h->num_sms, true);
   if (h->plan.cluster && !panel_cluster_fits<T>(h->plan))
     h->plan = plan_panel(g.M, bk, sizeof(T), h->num_sms, false);
@@ -478,7 +494,10 @@ cqr_status panel_kernel_step(cqr_handle h, int64_t kb, int bk, cudaStream_t st) 
   ensure_panel_plan<T>(h, bk);
   if (h->sub_bs > 0) return sub_panel_step<T>(h, kb, bk, st);
   ProfScope ps(h, K_PANEL, 1, st);
-  if (sizeof(T) == 4 && h->reg_ok) {
+  if (h->blk_ok) {
+    CK(launch_panel_blk<T>(h->blk, Q + kb * g.ldq, g.ldq, R + kb + kb * g.ldr, g.ldr, g.M, bk, h->tau,
+                           h->B.blk, h->B.status, (int)kb, st, h->wait_limit));
+  } else if (sizeof(T) == 4 && h->reg_ok) {
     CK(launch_panel_reg(h->reg_rpl, h->reg_cpw, h->reg_G, reinterpret_cast<float*>(Q + kb * g.ldq),
                         g.ldq, reinterpret_cast<float*>(R + kb + kb * g.ldr), g.ldr, g.M, bk, h->tau,
                         h->B.status, (int)kb, st, h->la_pdl && st == h->la_st[0], h->wait_limit));
@@ -570,7 +589,7 @@ bool lookahead_eligible(cqr_handle h) {
   if (env && env[0] == '0') return false;
   ensure_panel_plan<float>(h, (int)std::min<int64_t>(h->g.b, h->g.n));
   // a cooperative (grid-barrier) panel must not wait for CTAs of a concurrent GEMM
-  return h->reg_ok || h->plan.cluster;
+  return !h->blk_ok && (h->reg_ok || h->plan.cluster);
 }
 
 cqr_status lookahead_setup(cqr_handle h) {
@@ -1177,7 +1196,8 @@ cqr_status coded_qr_debug_bounds(int32_t* site) {
   return CQR_ENOTSUP;
 #else
   cudaError_t (*const takes[])(int*, int*) = {bounds_take_kernels, bounds_take_panel,
-                                              bounds_take_panel_reg, bounds_take_tc};
+                                              bounds_take_panel_reg, bounds_take_panel_blk,
+                                              bounds_take_tc};
   cqr_status out = CQR_OK;
   for (auto take : takes) {
     int code = 0, where = 0;

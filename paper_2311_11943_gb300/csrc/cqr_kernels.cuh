@@ -37,6 +37,14 @@ struct PanelPlan {
   size_t smem_bytes;
 };
 
+// Launch plan of the sub-block panel (cqr_panel_blk.cu).
+struct PanelBlkPlan {
+  int G;     // CTAs (cooperative)
+  int rpc;   // rows per CTA
+  int rs;    // column stride of a slice in shared memory
+  size_t smem_bytes;
+};
+
 template <typename T>
 cudaError_t launch_generator(int f, int p_r, int p_c, uint64_t seed, int gdist, double* Gt,
                              double* Gh, T* Gt_t, T* Gh_t, cudaStream_t st);
@@ -63,9 +71,20 @@ size_t panel_partial_bytes(int bk, size_t elem, int num_sms);
 cudaError_t bounds_take_kernels(int* code, int* site);
 cudaError_t bounds_take_panel(int* code, int* site);
 cudaError_t bounds_take_panel_reg(int* code, int* site);
+cudaError_t bounds_take_panel_blk(int* code, int* site);
 cudaError_t bounds_take_tc(int* code, int* site);
 // A guarded write past a four-element array (the bounds-checked build's self-test).
 cudaError_t launch_bounds_selftest(int idx, cudaStream_t st);
+
+// Sub-block panel (cqr_panel_blk.cu): false when the slices do not fit shared memory.  ws:
+// panel_blk_bytes of device memory, zero before the first launch and kept between launches; Q
+// 16-byte aligned with ldq a multiple of 16 bytes.
+bool plan_panel_blk(int64_t M, int bk, size_t elem, int num_sms, PanelBlkPlan* p);
+size_t panel_blk_bytes(int bk, size_t elem, int num_sms);
+template <typename T>
+cudaError_t launch_panel_blk(const PanelBlkPlan& p, T* Q, int64_t ldq, T* R, int64_t ldr, int64_t M,
+                             int bk, double tau, void* ws, int* status, int col0, cudaStream_t st,
+                             long long wait_limit);
 
 // Register-resident FP32 panel in one cluster (cqr_panel_reg.cu).
 bool plan_panel_reg(int64_t M, int bk, int* rpl, int* cpw, int* G);
