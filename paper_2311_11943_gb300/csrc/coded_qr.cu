@@ -27,7 +27,7 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-  size_t Q, R, Gt, Gh, Gt_t, Gh_t, Kpo, part, blk, bar, status, P, Rb, Pt, yw, xw, plans, cg, tc, total;
+  size_t Q, R, Gt, Gh, Gt_t, Gh_t, Kpo, part, blk, lsx, bar, status, P, Rb, Pt, yw, xw, plans, cg, tc, total;
 };
 
 struct Buffers {
@@ -40,6 +40,7 @@ struct Buffers {
   void* Kpo;  // (I_f + G~ G~^T)^{-1}: f x f doubles, then f x f in the storage type
   void* part;
   void* blk;  // sub-block panel: tag count, sums and partial sums
+  void* lsx;  // least squares by refinement: the same
   unsigned* bar;
   int* status;
   void* P;
@@ -130,6 +131,7 @@ Layout make_layout(const cqr_config* c, const Geo& g, int num_sms) {
   L.Kpo = take((size_t)kMaxF * kMaxF * (8 + s));
   L.part = take(panel_partial_bytes(bmax, s, num_sms));
   L.blk = take(panel_blk_bytes(bmax, s, num_sms));
+  L.lsx = take(g.f > 0 ? ls_refine_bytes(g.n, num_sms) : 256);
   L.bar = take(256);
   L.status = take(256);
   L.P = take((size_t)kMaxSplits * bmax * g.N * s);
@@ -279,6 +281,7 @@ cqr_status setup(cqr_handle h) {
   h->B.Kpo = base + L.Kpo;
   h->B.part = base + L.part;
   h->B.blk = base + L.blk;
+  h->B.lsx = base + L.lsx;
   h->B.bar = reinterpret_cast<unsigned*>(base + L.bar);
   h->B.status = reinterpret_cast<int*>(base + L.status);
   h->B.P = base + L.P;
@@ -806,6 +809,19 @@ cqr_status post_orth_y(cqr_handle h, const T* y, int64_t ldy, int32_t nrhs, T* y
 }
 
 // ------------------------------------------------------------------------------- solve
+// w = (I - Q_2^T Q_2)^{-1} Q_1^T y (or ... u) into w: by iterative refinement where its vectors
+// fit shared memory (n up to about 7000), else by conjugate gradients in FP64.
+template <typename T>
+cudaError_t ls_middle(cqr_handle h, const T* y, const T* u, T* w) {
+  const Geo& g = h->g;
+  bool taken = false;
+  const cudaError_t e = launch_ls_refine<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y, u, w,
+                                            h->B.cg, h->B.lsx, h->B.status, h->num_sms, h->st, &taken);
+  if (taken || e != cudaSuccess) return e;
+  return launch_ls_cg<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y, w, h->B.cg, h->B.bar,
+                         h->B.status, h->num_sms, h->st, u);
+}
+
 template <typename T>
 cqr_status solve_t(cqr_handle h, const T* y, int64_t ldy, T* x, int64_t ldx, int32_t nrhs) {
   const Geo& g = h->g;
@@ -816,8 +832,7 @@ cqr_status solve_t(cqr_handle h, const T* y, int64_t ldy, T* x, int64_t ldx, int
     for (int32_t k = 0; k < nrhs; ++k) {
       {
         ProfScope ps(h, K_SOLVE_GEMV, 1);
-        CK(launch_ls_cg<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y + (int64_t)k * ldy,
-                           x + (int64_t)k * ldx, h->B.cg, h->B.bar, h->B.status, h->num_sms, h->st));
+        CK(ls_middle<T>(h, y + (int64_t)k * ldy, nullptr, x + (int64_t)k * ldx));
       }
     }
     ProfScope ps(h, K_TRSV, nrhs);
@@ -1197,7 +1212,7 @@ cqr_status coded_qr_debug_bounds(int32_t* site) {
 #else
   cudaError_t (*const takes[])(int*, int*) = {bounds_take_kernels, bounds_take_panel,
                                               bounds_take_panel_reg, bounds_take_panel_blk,
-                                              bounds_take_tc};
+                                              bounds_take_lstsq, bounds_take_tc};
   cqr_status out = CQR_OK;
   for (auto take : takes) {
     int code = 0, where = 0;
@@ -1442,8 +1457,7 @@ cqr_status adjoint_lstsq_t(cqr_handle h, const T* A, int64_t lda, const T* y, in
     CK(launch_trsm_right<T>(0, R, g.ldr, n, u + (size_t)j * n, 1, 1, 1, h->st));
   // w = (I - Q_2^T Q_2)^{-1} u (FP64 conjugate gradients), z = R^{-1} w
   for (int32_t j = 0; j < k; ++j)
-    CK(launch_ls_cg<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, n, nullptr, w + (size_t)j * n,
-                       h->B.cg, h->B.bar, h->B.status, h->num_sms, h->st, u + (size_t)j * n));
+    CK(ls_middle<T>(h, nullptr, u + (size_t)j * n, w + (size_t)j * n));
   for (int32_t j = 0; j < k; ++j)
     CK(launch_trsm_right<T>(1, R, g.ldr, n, w + (size_t)j * n, 1, 1, 1, h->st));
   const T* z = w;

@@ -72,6 +72,7 @@ cudaError_t bounds_take_kernels(int* code, int* site);
 cudaError_t bounds_take_panel(int* code, int* site);
 cudaError_t bounds_take_panel_reg(int* code, int* site);
 cudaError_t bounds_take_panel_blk(int* code, int* site);
+cudaError_t bounds_take_lstsq(int* code, int* site);
 cudaError_t bounds_take_tc(int* code, int* site);
 // A guarded write past a four-element array (the bounds-checked build's self-test).
 cudaError_t launch_bounds_selftest(int idx, cudaStream_t st);
@@ -168,6 +169,15 @@ template <typename T>
 cudaError_t launch_ls_cg(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, int64_t c, int64_t n,
                          const T* y, T* x, double* ws, unsigned* bar, int* status, int num_sms,
                          cudaStream_t st, const T* u = nullptr);
+
+// The same by iterative refinement (cqr_lstsq.cu); *taken false (nothing launched) when its
+// vectors do not fit shared memory.  z: n doubles of workspace; xws: ls_refine_bytes of device
+// memory, zero before the first launch and kept between launches.
+size_t ls_refine_bytes(int64_t n, int num_sms);
+template <typename T>
+cudaError_t launch_ls_refine(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, int64_t c, int64_t n,
+                             const T* y, const T* u, T* x, double* z, void* xws, int* status,
+                             int num_sms, cudaStream_t st, bool* taken);
 
 // ---------------------------------------------------------------- adjoint building blocks
 // C (M x N) = alpha op(A) op(B) + beta C (op = transpose when ta / tb); beta == 0 ignores C.
