@@ -27,7 +27,7 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-  size_t Q, R, Gt, Gh, Gt_t, Gh_t, Kpo, part, blk, lsx, bar, status, P, Rb, Pt, yw, xw, plans, cg, tc, total;
+  size_t Q, R, Gt, Gh, Gt_t, Gh_t, Kpo, part, blk, lsx, bar, status, P, Rb, Pt, yw, xw, plans, cg, tc, f64, total;
 };
 
 struct Buffers {
@@ -51,6 +51,7 @@ struct Buffers {
   DecodePlan* plans;
   double* cg;
   void* tc;
+  void* f64;  // FP64 update by integer slices: operand digits
 };
 
 // Checksum blocks per code.  Out-of-node storage: f (one per tolerated failure, on f extra
@@ -144,6 +145,7 @@ Layout make_layout(const cqr_config* c, const Geo& g, int num_sms) {
   L.tc = take(c->dtype == CQR_F32 && c->mma != CQR_MMA_SIMT
                   ? tc_workspace_bytes(c->mma, g.M, g.N, g.n, bmax, c->reorth_block != 0)
                   : 0);
+  L.f64 = take(c->dtype == CQR_F64 ? f64_gemm_bytes(g.M, g.N, bmax) : 0);
   L.total = off;
   return L;
 }
@@ -189,6 +191,7 @@ struct cqr_handle_s {
   size_t esz = 8;
   double tau = 0.7071067811865476;
   TcGemm* tc = nullptr;
+  F64Gemm* f64 = nullptr;
   PanelPlan plan{};
   int plan_bk = -1;
   bool reg_ok = false;
@@ -292,6 +295,7 @@ cqr_status setup(cqr_handle h) {
   h->B.plans = reinterpret_cast<DecodePlan*>(base + L.plans);
   h->B.cg = reinterpret_cast<double*>(base + L.cg);
   h->B.tc = base + L.tc;
+  h->B.f64 = base + L.f64;
   h->mask.assign((size_t)h->g.grid_rows * h->g.grid_cols, 0);
   CK(cudaMallocHost(&h->plans_host, sizeof(DecodePlan) * (size_t)(h->g.grid_cols + h->g.p_c + h->g.f + 2)));
   CK(cudaMallocHost(&h->status_host, 4 * sizeof(int)));
@@ -304,6 +308,11 @@ cqr_status setup(cqr_handle h) {
                       h->st);
     if (!h->tc) return CQR_ECUDA;
     tc_set_status(h->tc, h->B.status);
+  }
+  const int64_t bmax = std::min<int64_t>(h->cfg.b, h->g.n);
+  if (h->cfg.dtype == CQR_F64 && f64_gemm_bytes(h->g.M, h->g.N, bmax) > 0) {
+    h->f64 = f64_gemm_create(h->g.M, h->g.N, bmax, h->B.f64, h->num_sms);
+    if (!h->f64) return CQR_ECUDA;
   }
   return CQR_OK;
 }
@@ -533,6 +542,35 @@ cqr_status tc_update_cols(cqr_handle h, int64_t kb, int bk, int64_t j0, int64_t 
   return CQR_OK;
 }
 
+// FP64 trailing update by integer slices, in blocks of the columns whose digits are held.
+cqr_status f64_update(cqr_handle h, int64_t kb, int bk, int64_t j0, int64_t w) {
+  const Geo& g = h->g;
+  double* Q = ptr<double>(h->B.Q);
+  double* R = ptr<double>(h->B.R);
+  double* P = ptr<double>(h->B.P);
+  double* Rb = ptr<double>(h->B.Rb);
+  {
+    ProfScope ps(h, K_TC_SPLIT, 2);
+    CK(f64_gemm_panel(h->f64, Q + kb * g.ldq, g.ldq, bk, h->st));
+  }
+  const int64_t cols = f64_gemm_cols(h->f64);
+  for (int64_t c0 = 0; c0 < w; c0 += cols) {
+    const int64_t wc = std::min(cols, w - c0), j = j0 + c0;
+    int splits = 0;
+    {
+      ProfScope ps(h, K_TC_RBAR, 2);
+      CK(f64_gemm_rbar(h->f64, Q + j * g.ldq, g.ldq, wc, bk, P, &splits, h->B.status, h->st));
+    }
+    {
+      ProfScope ps(h, K_SPLITK_REDUCE, 1);
+      CK(launch_splitk_reduce<double>(P, splits, bk, wc, R + kb + j * g.ldr, g.ldr, Rb, h->st));
+    }
+    ProfScope ps(h, K_TC_UPDATE, 2);
+    CK(f64_gemm_update(h->f64, Rb, wc, bk, Q + j * g.ldq, g.ldq, h->B.status, h->st));
+  }
+  return CQR_OK;
+}
+
 // One panel in stream order: block reorthogonalisation, panel, trailing update of every
 // column to the right.
 template <typename T>
@@ -557,6 +595,8 @@ cqr_status panel_step(cqr_handle h, int t) {
     }
     return tc_update_cols(h, kb, bk, j0, w, buf, 0, 0, h->st);
   }
+  if constexpr (sizeof(T) == 8)
+    if (h->f64 && f64_gemm_pays(g.M, w, bk)) return f64_update(h, kb, bk, j0, w);
   const int splits = choose_splits(bk, w, g.M, h->num_sms);
   {
     ProfScope ps(h, K_GEMM_RBAR, 1);
@@ -896,6 +936,7 @@ cqr_status coded_qr_destroy(cqr_handle h) {
   if (!h) return CQR_OK;
   if (h->st || true) cudaStreamSynchronize(h->st);
   if (h->tc) tc_destroy(h->tc);
+  if (h->f64) f64_gemm_destroy(h->f64);
   for (auto e : h->la_ev)
     if (e) cudaEventDestroy(e);
   for (auto q : h->la_st)
@@ -1212,7 +1253,8 @@ cqr_status coded_qr_debug_bounds(int32_t* site) {
 #else
   cudaError_t (*const takes[])(int*, int*) = {bounds_take_kernels, bounds_take_panel,
                                               bounds_take_panel_reg, bounds_take_panel_blk,
-                                              bounds_take_lstsq, bounds_take_tc};
+                                              bounds_take_lstsq, bounds_take_f64_gemm,
+                                              bounds_take_tc};
   cqr_status out = CQR_OK;
   for (auto take : takes) {
     int code = 0, where = 0;

@@ -73,6 +73,7 @@ cudaError_t bounds_take_panel(int* code, int* site);
 cudaError_t bounds_take_panel_reg(int* code, int* site);
 cudaError_t bounds_take_panel_blk(int* code, int* site);
 cudaError_t bounds_take_lstsq(int* code, int* site);
+cudaError_t bounds_take_f64_gemm(int* code, int* site);
 cudaError_t bounds_take_tc(int* code, int* site);
 // A guarded write past a four-element array (the bounds-checked build's self-test).
 cudaError_t launch_bounds_selftest(int idx, cudaStream_t st);
@@ -125,6 +126,25 @@ cudaError_t launch_splitk_reduce(const T* P, int splits, int bk, int64_t w, T* R
 template <typename T>
 cudaError_t launch_gemm_nn_sub(const T* A, int64_t lda, const T* B, int64_t ldb, T* C,
                                int64_t ldc, int64_t M, int bk, int64_t w, cudaStream_t st);
+
+// The FP64 trailing update on the BF16 tensor cores by exact integer slices (cqr_f64_gemm.cu), for
+// updates large enough: the panel's digits, then per block of at most f64_gemm_cols columns the
+// partials of Rbar (summed by launch_splitk_reduce) and C -= Qbar Rb.
+// Whether an update of w columns by bk of M rows gains: each of its launches takes some
+// microseconds and a tile 128 x 64 outputs, the CUDA cores about 0.6 T products per second.
+inline bool f64_gemm_pays(int64_t M, int64_t w, int64_t bk) {
+  return w >= 64 && bk >= 16 && (double)M * (double)w * (double)bk >= 2.5e7;
+}
+struct F64Gemm;
+size_t f64_gemm_bytes(int64_t M, int64_t N, int64_t b);  // workspace; 0: not for this problem
+F64Gemm* f64_gemm_create(int64_t M, int64_t N, int64_t b, void* ws, int num_sms);
+void f64_gemm_destroy(F64Gemm* t);
+int64_t f64_gemm_cols(const F64Gemm* t);
+cudaError_t f64_gemm_panel(F64Gemm* t, const double* Q, int64_t ldq, int bk, cudaStream_t st);
+cudaError_t f64_gemm_rbar(F64Gemm* t, const double* B, int64_t ldb, int64_t w, int bk, double* P,
+                          int* splits, int* status, cudaStream_t st);
+cudaError_t f64_gemm_update(F64Gemm* t, const double* Rb, int64_t w, int bk, double* C, int64_t ldc,
+                            int* status, cudaStream_t st);
 
 template <typename T>
 cudaError_t launch_poison(const Geo& g, const int* tiles, int count, T* Q, T* R,
