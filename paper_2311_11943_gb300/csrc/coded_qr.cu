@@ -380,12 +380,15 @@ cqr_status encode_t(cqr_handle h, const T* A, int64_t lda) {
 }
 
 // ------------------------------------------------------------------------------- factor
-int choose_splits(int bk, int64_t w, int64_t K, int num_sms) {
-  const int64_t tiles = ((bk + 63) / 64) * ((w + 63) / 64);
+// Splits over K of a CUDA-core Rbar product: enough 64 x 64 tiles for two per SM, chunks of 256 at
+// least; in FP64 enough 32 x 32 tiles (launch_gemm_tn_splitk), chunks of 32 at least.
+int choose_splits(int bk, int64_t w, int64_t K, int num_sms, size_t elem) {
+  const int t = elem == 8 ? 32 : 64, least = elem == 8 ? 32 : 256;
+  const int64_t tiles = ((bk + t - 1) / t) * ((w + t - 1) / t);
   int s = (int)((2 * num_sms + tiles - 1) / tiles);
   if (s > kMaxSplits) s = kMaxSplits;
   if (s < 1) s = 1;
-  while (s > 1 && K / s < 256) --s;
+  while (s > 1 && K / s < least) --s;
   return s;
 }
 
@@ -459,7 +462,7 @@ cqr_status sub_panel_step(cqr_handle h, int64_t kb, int bk, cudaStream_t st) {
     const int64_t w = kb + bk - j0;
     if (w <= 0) break;
     ProfScope ps(h, K_PANEL_SUB_UPDATE, 3, st);
-    const int splits = choose_splits(w0, w, g.M, h->num_sms);
+    const int splits = choose_splits(w0, w, g.M, h->num_sms, sizeof(T));
     CK(launch_gemm_tn_splitk<T>(Q + ks * g.ldq, g.ldq, Q + j0 * g.ldq, g.ldq, g.M, w0, w, splits,
                                 ptr<T>(h->B.P), st));
     CK(launch_splitk_reduce<T>(ptr<T>(h->B.P), splits, w0, w, R + ks + j0 * g.ldr, g.ldr,
@@ -487,7 +490,7 @@ cqr_status reorth_block_step(cqr_handle h, int64_t kb, int bk, int buf, cudaStre
     return CQR_OK;
   }
   ProfScope ps(h, K_BLOCK_REORTH, 3, st);
-  const int sp = choose_splits((int)kb, bk, g.M, h->num_sms);
+  const int sp = choose_splits((int)kb, bk, g.M, h->num_sms, sizeof(T));
   CK(launch_gemm_tn_splitk<T>(Q, g.ldq, Q + kb * g.ldq, g.ldq, g.M, (int)kb, bk, sp,
                               ptr<T>(h->B.P), st));
   CK(launch_splitk_reduce<T>(ptr<T>(h->B.P), sp, (int)kb, bk, R + kb * g.ldr, g.ldr,
@@ -597,7 +600,7 @@ cqr_status panel_step(cqr_handle h, int t) {
   }
   if constexpr (sizeof(T) == 8)
     if (h->f64 && f64_gemm_pays(g.M, w, bk)) return f64_update(h, kb, bk, j0, w);
-  const int splits = choose_splits(bk, w, g.M, h->num_sms);
+  const int splits = choose_splits(bk, w, g.M, h->num_sms, sizeof(T));
   {
     ProfScope ps(h, K_GEMM_RBAR, 1);
     CK(launch_gemm_tn_splitk<T>(Q + kb * g.ldq, g.ldq, Q + j0 * g.ldq, g.ldq, g.M, bk, w, splits,

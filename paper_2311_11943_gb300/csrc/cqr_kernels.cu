@@ -303,31 +303,42 @@ cudaError_t launch_encode(const Geo& g, const T* A, int64_t lda, const T* Gt, co
 
 // ===================================================================== a4/a5 SIMT GEMMs
 // Rbar = Qbar^T Qtrail (split over K) and Qtrail -= Qbar Rbar on CUDA cores: the FP64 path
-// and the FP32 reference path.  64 x 64 output tiles, 256 threads, 4 x 4 per thread with a
-// stride-16 micro-tile so that each half-warp touches 16 consecutive rows.
+// and the FP32 reference path.  TILE x TILE output tiles (64, or 32), 256 threads, E x E
+// (E = TILE / 16) per thread with a stride-16 micro-tile so that each half-warp touches 16
+// consecutive rows.  Tiles of 32 where those of 64 would leave SMs idle: FP64 runs at two products
+// per cycle and SM, so an SM without a tile is what a small update costs (FP64, 320 x 288 by 32:
+// Rbar 338 us on 5 CTAs of 64 x 64 before); FP32 only where three quarters of the SMs would idle,
+// since a tile of 32 reads twice as much per product.
 template <typename T>
+bool small_tiles(int64_t rows, int64_t cols, int64_t splits) {
+  const int64_t n64 = ((rows + 63) / 64) * ((cols + 63) / 64) * splits;
+  return n64 < (sizeof(T) == 8 ? 300 : 38);
+}
+
+template <typename T, int TILE>
 __global__ void __launch_bounds__(256) k_gemm_tn_splitk(const T* __restrict__ A, int64_t lda,
                                                          const T* __restrict__ B, int64_t ldb,
                                                          int64_t K, int bk, int64_t w,
                                                          int64_t kchunk, T* __restrict__ P) {
-  __shared__ T As[32][65];
-  __shared__ T Bs[32][65];
+  constexpr int E = TILE / 16;
+  __shared__ T As[32][TILE + 1];
+  __shared__ T Bs[32][TILE + 1];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   CQR_CHECK(lda >= K && ldb >= K, 103);  // uniform over the launch: before any barrier
-  const int i0 = blockIdx.x * 64;
-  const int64_t j0 = (int64_t)blockIdx.y * 64;
+  const int i0 = blockIdx.x * TILE;
+  const int64_t j0 = (int64_t)blockIdx.y * TILE;
   const int64_t k0 = (int64_t)blockIdx.z * kchunk;
   const int64_t k1 = (k0 + kchunk < K) ? k0 + kchunk : K;
-  T acc[4][4];
+  T acc[E][E];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < E; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+    for (int b = 0; b < E; ++b) acc[a][b] = T(0);
   for (int64_t kb = k0; kb < k1; kb += 32) {
     const int kk = tid & 31;
     const int64_t k = kb + kk;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
+    for (int e = 0; e < TILE / 8; ++e) {
       const int ii = (tid >> 5) + 8 * e;
       const int i = i0 + ii;
       As[kk][ii] = (k < k1 && i < bk) ? A[k + (int64_t)i * lda] : T(0);
@@ -337,21 +348,21 @@ __global__ void __launch_bounds__(256) k_gemm_tn_splitk(const T* __restrict__ A,
     __syncthreads();
 #pragma unroll 8
     for (int q = 0; q < 32; ++q) {
-      T a[4], b[4];
+      T a[E], b[E];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) { a[e] = As[q][tx + 16 * e]; b[e] = Bs[q][ty + 16 * e]; }
+      for (int e = 0; e < E; ++e) { a[e] = As[q][tx + 16 * e]; b[e] = Bs[q][ty + 16 * e]; }
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < E; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
+        for (int y = 0; y < E; ++y) acc[x][y] += a[x] * b[y];
     }
     __syncthreads();
   }
   T* Ps = P + (size_t)blockIdx.z * (size_t)bk * (size_t)w;
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < E; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
+    for (int y = 0; y < E; ++y) {
       const int i = i0 + tx + 16 * x;
       const int64_t j = j0 + ty + 16 * y;
       if (i < bk && j < w) Ps[i + j * bk] = acc[x][y];
@@ -363,8 +374,12 @@ cudaError_t launch_gemm_tn_splitk(const T* A, int64_t lda, const T* B, int64_t l
                                   int bk, int64_t w, int splits, T* P, cudaStream_t st) {
   int64_t kchunk = (K + splits - 1) / splits;
   kchunk = (kchunk + 31) / 32 * 32;
-  dim3 grd((unsigned)((bk + 63) / 64), (unsigned)((w + 63) / 64), (unsigned)splits);
-  k_gemm_tn_splitk<T><<<grd, 256, 0, st>>>(A, lda, B, ldb, K, bk, w, kchunk, P);
+  const int tile = small_tiles<T>(bk, w, splits) ? 32 : 64;
+  dim3 grd((unsigned)((bk + tile - 1) / tile), (unsigned)((w + tile - 1) / tile), (unsigned)splits);
+  if (tile == 32)
+    k_gemm_tn_splitk<T, 32><<<grd, 256, 0, st>>>(A, lda, B, ldb, K, bk, w, kchunk, P);
+  else
+    k_gemm_tn_splitk<T, 64><<<grd, 256, 0, st>>>(A, lda, B, ldb, K, bk, w, kchunk, P);
   return cudaGetLastError();
 }
 
@@ -398,26 +413,27 @@ cudaError_t launch_splitk_reduce(const T* P, int splits, int bk, int64_t w, T* R
   return cudaGetLastError();
 }
 
-template <typename T>
+template <typename T, int TILE>
 __global__ void __launch_bounds__(256) k_gemm_nn_sub(const T* __restrict__ A, int64_t lda,
                                                       const T* __restrict__ B, int64_t ldb,
                                                       T* __restrict__ C, int64_t ldc, int64_t M,
                                                       int bk, int64_t w) {
-  __shared__ T As[32][65];
-  __shared__ T Bs[32][65];
+  constexpr int E = TILE / 16;
+  __shared__ T As[32][TILE + 1];
+  __shared__ T Bs[32][TILE + 1];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   CQR_CHECK(lda >= M && ldc >= M && ldb >= bk, 105);  // uniform: before any barrier
-  const int64_t i0 = (int64_t)blockIdx.x * 64;
-  const int64_t j0 = (int64_t)blockIdx.y * 64;
-  T acc[4][4];
+  const int64_t i0 = (int64_t)blockIdx.x * TILE;
+  const int64_t j0 = (int64_t)blockIdx.y * TILE;
+  T acc[E][E];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < E; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+    for (int b = 0; b < E; ++b) acc[a][b] = T(0);
   for (int kb = 0; kb < bk; kb += 32) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int ii = tid & 63, kk = (tid >> 6) + 4 * e;
+    for (int e = 0; e < TILE / 8; ++e) {
+      const int ii = tid % TILE, kk = tid / TILE + 256 / TILE * e;
       const int64_t i = i0 + ii;
       const int k = kb + kk;
       As[kk][ii] = (i < M && k < bk) ? A[i + (int64_t)k * lda] : T(0);
@@ -429,20 +445,20 @@ __global__ void __launch_bounds__(256) k_gemm_nn_sub(const T* __restrict__ A, in
     __syncthreads();
 #pragma unroll 8
     for (int q = 0; q < 32; ++q) {
-      T a[4], b[4];
+      T a[E], b[E];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) { a[e] = As[q][tx + 16 * e]; b[e] = Bs[q][ty + 16 * e]; }
+      for (int e = 0; e < E; ++e) { a[e] = As[q][tx + 16 * e]; b[e] = Bs[q][ty + 16 * e]; }
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < E; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
+        for (int y = 0; y < E; ++y) acc[x][y] += a[x] * b[y];
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < E; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
+    for (int y = 0; y < E; ++y) {
       const int64_t i = i0 + tx + 16 * x;
       const int64_t j = j0 + ty + 16 * y;
       if (i < M && j < w) C[i + j * ldc] -= acc[x][y];
@@ -452,8 +468,12 @@ __global__ void __launch_bounds__(256) k_gemm_nn_sub(const T* __restrict__ A, in
 template <typename T>
 cudaError_t launch_gemm_nn_sub(const T* A, int64_t lda, const T* B, int64_t ldb, T* C,
                                int64_t ldc, int64_t M, int bk, int64_t w, cudaStream_t st) {
-  dim3 grd((unsigned)((M + 63) / 64), (unsigned)((w + 63) / 64));
-  k_gemm_nn_sub<T><<<grd, 256, 0, st>>>(A, lda, B, ldb, C, ldc, M, bk, w);
+  const int tile = small_tiles<T>(M, w, 1) ? 32 : 64;
+  dim3 grd((unsigned)((M + tile - 1) / tile), (unsigned)((w + tile - 1) / tile));
+  if (tile == 32)
+    k_gemm_nn_sub<T, 32><<<grd, 256, 0, st>>>(A, lda, B, ldb, C, ldc, M, bk, w);
+  else
+    k_gemm_nn_sub<T, 64><<<grd, 256, 0, st>>>(A, lda, B, ldb, C, ldc, M, bk, w);
   return cudaGetLastError();
 }
 
