@@ -186,8 +186,9 @@ __device__ __forceinline__ void gram(const Blk<T>& c, int jx, int n, int a0, int
   using V = Vec<T>;
   const int na = (w + 3) / 4;
   const int ntiles = (S / 4) * na;
+  // FP64: at most four lanes, since a lane without rows takes its share of the FP64 pipe too
   int lks = 0;
-  while (lks < 5 && (2 << lks) * ntiles <= kNT) ++lks;
+  while (lks < (sizeof(T) == 4 ? 5 : 2) && (2 << lks) * ntiles <= kNT) ++lks;
   const int ks = 1 << lks;
   const int kg = threadIdx.x & (ks - 1);
   const T* bx = c.P + (size_t)jx * c.rs;
