@@ -656,7 +656,7 @@ cqr_status factor_lookahead(cqr_handle h, int t0, int t1) {
   // programmatic dependent launch along the critical stream (CQR_PDL=0 turns it off)
   const char* pe = getenv("CQR_PDL");
   h->la_pdl = !(pe && pe[0] == '0');
-  tc_set_pdl_stream(h->tc, h->la_pdl ? A : nullptr);
+  tc_set_pdl_stream(h->tc, h->la_pdl, A);
   cudaEvent_t ev_fork = h->la_ev[0], ev_a = h->la_ev[1], ev_w = h->la_ev[2];
   CK(cudaEventRecord(ev_fork, h->st));
   CK(cudaStreamWaitEvent(A, ev_fork, 0));  // B joins through A's events (only if it gets work)
@@ -1001,6 +1001,13 @@ cqr_status coded_qr_factor(cqr_handle h, int32_t t0, int32_t t1) {
     if (s != CQR_OK) return s;
     h->panels_run += t1 - t0;
   } else {
+    // programmatic dependent launch of the tensor-core kernels along the handle's stream: each
+    // starts while its predecessor finishes and waits for it before it touches data (4096^2:
+    // nine launches per panel of a quarter of a millisecond)
+    if (h->tc) {
+      const char* pe = getenv("CQR_PDL");
+      tc_set_pdl_stream(h->tc, !(pe && pe[0] == '0'), h->st);
+    }
     for (int t = t0; t < t1; ++t) {
       cqr_status s = h->esz == 8 ? panel_step<double>(h, t) : panel_step<float>(h, t);
       if (s != CQR_OK) return s;

@@ -628,7 +628,8 @@ struct TcGemm {
   int64_t n, ldrow;
   int num_sms;
   int* status;
-  cudaStream_t pdl_st = nullptr;  // launches on this stream use programmatic dependent launch
+  bool pdl = false;  // launches on pdl_st use programmatic dependent launch
+  cudaStream_t pdl_st = nullptr;
   CUtensorMap tm_q_b;        // Q (FP32) as GEMM1's raw B (box 32 x BN)
   CUtensorMap tm_ak[2][2];   // [buffer][plane] panel, column-major (box KE x BM)
   CUtensorMap tm_at[2][2];   // [buffer][plane] panel, row-major (box KE x BM)
@@ -736,7 +737,7 @@ cudaError_t launch_mode(const TcGemm* t, bool split, const TcMaps& maps, const T
                         cudaStream_t st, int max_ctas = 0) {
   const bool three = t->nplanes == 2;
   const int mc = max_ctas > 0 ? std::min(max_ctas, t->num_sms) : t->num_sms;
-  const bool pdl = st == t->pdl_st && st != nullptr;
+  const bool pdl = t->pdl && st == t->pdl_st;
   if (!t->bf) {
     if (pair_m_tiles(three, false, split, job.m_tiles))
       return launch_gemm<false, 2, 2, 2, 2>(maps, job, mc, st, pdl);
@@ -857,7 +858,10 @@ void tc_destroy(TcGemm* t) { delete t; }
 
 void tc_set_status(TcGemm* t, int* status) { t->status = status; }
 
-void tc_set_pdl_stream(TcGemm* t, cudaStream_t st) { t->pdl_st = st; }
+void tc_set_pdl_stream(TcGemm* t, bool on, cudaStream_t st) {
+  t->pdl = on;
+  t->pdl_st = st;
+}
 
 namespace {
 // Split-K factor of a product with m1 x n1 output tiles and K = M rows: the count s whose
@@ -900,7 +904,7 @@ cudaError_t tc_split_panel(TcGemm* t, int64_t kb, int bk, bool finished, int buf
   const int m1 = (bk + BM - 1) / BM;
   dim3 grd((unsigned)((t->M + 31) / 32), (unsigned)((std::max(bkp, m1 * BM) + 31) / 32));
   void* qh = finished ? t->Qr_hi : nullptr;
-  const bool pdl = st == t->pdl_st && st != nullptr;
+  const bool pdl = t->pdl && st == t->pdl_st;
   const float* q0 = t->Q + kb * t->ldq;
   if (t->bf) {
     using B16 = __nv_bfloat16;
@@ -979,7 +983,7 @@ cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, floa
   const int splits = tc_splits(t, m1, n1, &kchunk, max_ctas);
   const int64_t total = (int64_t)bkp * w;
   const int blocks = (int)std::min<int64_t>(4096, (total + 255) / 256);
-  const bool pdl = st == t->pdl_st && st != nullptr;
+  const bool pdl = t->pdl && st == t->pdl_st;
   const float* P = t->P[ctx];
   float* Rd = R + kb + j0 * ldr;
   if (t->bf)
@@ -1047,7 +1051,7 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
   const int64_t kbp = round_to(kb, KE);
   {
     const dim3 blocks((unsigned)((bk + 31) / 32), (unsigned)((kbp + 31) / 32));
-    const bool pdl = st == t->pdl_st && st != nullptr;
+    const bool pdl = t->pdl && st == t->pdl_st;
     const float* P0 = t->P[0];
     if (t->bf)
       e = launch_k(k_tc_reduce_t<__nv_bfloat16>, blocks, dim3(256), 0, st, pdl, P0, splits,
@@ -1107,7 +1111,7 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
   *launches = 5;
   const int64_t total = t->M * (int64_t)bk;
   const int blocks = (int)std::min<int64_t>((int64_t)t->num_sms * 8, (total + 255) / 256);
-  const bool pdl = st == t->pdl_st && st != nullptr;
+  const bool pdl = t->pdl && st == t->pdl_st;
   return launch_k(k_tc_sub_partials, dim3(blocks), dim3(256), 0, st, pdl, (const float*)t->P[0], splits2,
                   t->M, (int64_t)bk, t->Q + kb * t->ldq, t->ldq);
 }
