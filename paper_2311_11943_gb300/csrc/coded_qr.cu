@@ -1264,6 +1264,7 @@ cqr_status coded_qr_debug_bounds(int32_t* site) {
   cudaError_t (*const takes[])(int*, int*) = {bounds_take_kernels, bounds_take_panel,
                                               bounds_take_panel_reg, bounds_take_panel_blk,
                                               bounds_take_lstsq, bounds_take_f64_gemm,
+                                              bounds_take_adjoint,
                                               bounds_take_tc};
   cqr_status out = CQR_OK;
   for (auto take : takes) {
@@ -1436,13 +1437,22 @@ cqr_status adjoint_qr_t(cqr_handle h, const T* Q, int64_t ldq, const T* Qbar, in
   bool tcq = false;
   if constexpr (sizeof(T) == 4) tcq = h->tc != nullptr;
   const size_t base_el = (2 * nn + (size_t)mp * n + 63) / 64 * 64;
-  const size_t plane_el = tcq ? std::max(tc_gemm_sub_planes(true, n, mp), tc_gemm_sub_planes(false, mp, n)) : 0;
-  cqr_status s = adj_scratch(h, sizeof(T) * (base_el + plane_el));
+  const size_t plane_el = tcq ? std::max({tc_gemm_sub_planes(true, n, mp), tc_gemm_sub_planes(false, mp, n),
+                                          tc_gemm_sub_planes(false, n, n)}) : 0;
+  // the triangular solve on the tensor cores: R^T (ld nt), the inverses of R's diagonal blocks
+  // and one block of X
+  const int ib = tri_inverse_block();
+  const int64_t nt = round_up(n, 4), nblk = (n + ib - 1) / ib;
+  const size_t tri_el = tcq ? round_up((size_t)nt * n + (size_t)nblk * ib * ib + (size_t)mp * ib, 64) : 0;
+  cqr_status s = adj_scratch(h, sizeof(T) * (base_el + tri_el + plane_el));
   if (s != CQR_OK) return s;
   T* Mm = static_cast<T*>(h->adj);
   T* S = Mm + nn;
   T* Bb = S + nn;
-  float* planes = reinterpret_cast<float*>(Mm + base_el);
+  T* Rt = Mm + base_el;
+  T* Vi = Rt + (size_t)nt * n;
+  T* Xb = Vi + (size_t)nblk * ib * ib;
+  float* planes = reinterpret_cast<float*>(Mm + base_el + tri_el);
   const T* R = ptr<T>(h->B.R);
   // C -= op(A) B on the tensor cores; false when the operands break a tensor-map rule
   auto tc_sub = [&](bool a_trans, const T* A_, int64_t lda_, const T* B_, int64_t ldb_, T* C_,
@@ -1457,9 +1467,17 @@ cqr_status adjoint_qr_t(cqr_handle h, const T* Q, int64_t ldq, const T* Qbar, in
     return e == cudaErrorInvalidValue ? 0 : -1;
   };
   // M = R Rbar^T - Qbar^T Q
-  if (Rbar)
+  bool rr = false;
+  if (Rbar && tcq) {  // 0 - R (-Rbar^T)
+    CK(launch_axpy2d<T>(n, n, T(-1), Rbar, ldrb, 1, Rt, 1, nt, true, h->st));
+    CK(cudaMemsetAsync(Mm, 0, sizeof(T) * nn, h->st));
+    const int r = tc_sub(false, R, g.ldr, Rt, nt, Mm, n, n, n, n);
+    if (r < 0) return CQR_ECUDA;
+    rr = r > 0;
+  }
+  if (Rbar && !rr)
     CK(launch_gemm_general<T>(0, 1, n, n, n, T(1), R, g.ldr, Rbar, ldrb, T(0), Mm, n, h->st));
-  else
+  else if (!Rbar)
     CK(cudaMemsetAsync(Mm, 0, sizeof(T) * nn, h->st));
   if (Qbar) {
     const int r = tc_sub(true, Qbar, ldqb, Q, ldq, Mm, n, n, n, mp);
@@ -1483,7 +1501,31 @@ cqr_status adjoint_qr_t(cqr_handle h, const T* Q, int64_t ldq, const T* Qbar, in
   }
   if (r3 == 0)
     CK(launch_gemm_general<T>(0, 0, mp, n, n, T(1), Q, ldq, S, n, T(1), Bb, mp, h->st));
-  CK(launch_trsm_right<T>(1, R, g.ldr, n, Bb, 1, mp, mp, h->st));
+  bool solved = false;
+  if constexpr (sizeof(T) == 4) {
+    if (tcq && n > ib) {
+      // Bbar R^{-T} by blocks of ib columns from the last: X = B U^{-T} with the inverse of the
+      // diagonal block, then every earlier column less X times its rows of R^T in 3xTF32
+      // (8192 x 1024: 16 row-block solves of 60 us and as many CUDA-core products of 23 to 76 us
+      // before)
+      CK(launch_axpy2d<T>(n, n, T(1), R, g.ldr, 1, Rt, 1, nt, true, h->st));
+      CK(launch_tri_inverse<T>(R, g.ldr, n, Vi, h->st));
+      solved = true;
+      for (int64_t J = nblk - 1; J >= 0 && solved; --J) {
+        const int64_t j0 = J * ib, jb = std::min<int64_t>(ib, n - j0);
+        CK(launch_gemm_general<T>(0, 1, mp, jb, jb, T(1), Bb + j0 * mp, mp, Vi + J * ib * ib, ib, T(0),
+                                  Xb, mp, h->st));
+        CK(launch_axpy2d<T>(mp, jb, T(1), Xb, 1, mp, Bb + j0 * mp, 1, mp, true, h->st));
+        if (j0 > 0) {
+          const int r = tc_sub(false, Xb, mp, Rt + j0, nt, Bb, mp, mp, j0, jb);
+          if (r < 0) return CQR_ECUDA;
+          if (r == 0)
+            CK(launch_gemm_general<T>(0, 0, mp, j0, jb, T(-1), Xb, mp, Rt + j0, nt, T(1), Bb, mp, h->st));
+        }
+      }
+    }
+  }
+  if (!solved) CK(launch_trsm_right<T>(1, R, g.ldr, n, Bb, 1, mp, mp, h->st));
   // Abar += G_0^T Bbar (G_0 is symmetric: its leading block I - V V^T / 2 is), rows < m
   if (g.f > 0) CK(launch_post_orth<T>(g, ptr<T>(h->B.Gt_t), Bb, mp, mp, n, Bb, mp, h->st));
   CK(launch_axpy2d<T>(g.m, n, T(1), Bb, 1, mp, Abar, 1, ldab, false, h->st));
@@ -1505,23 +1547,18 @@ cqr_status adjoint_lstsq_t(cqr_handle h, const T* A, int64_t lda, const T* y, in
   const T* R = ptr<T>(h->B.R);
   // u = R^{-T} xbar: rows of the (k x n) view solve u^T R = xbar^T
   CK(launch_axpy2d<T>(n, k, T(1), xbar, 1, ldxb, u, 1, n, true, h->st));
-  for (int32_t j = 0; j < k; ++j)  // each right-hand side is one contiguous row
-    CK(launch_trsm_right<T>(0, R, g.ldr, n, u + (size_t)j * n, 1, 1, 1, h->st));
+  CK(launch_trsv_upper_t<T>(R, g.ldr, n, u, n, k, h->st));
   // w = (I - Q_2^T Q_2)^{-1} u (FP64 conjugate gradients), z = R^{-1} w
   for (int32_t j = 0; j < k; ++j)
     CK(ls_middle<T>(h, nullptr, u + (size_t)j * n, w + (size_t)j * n));
-  for (int32_t j = 0; j < k; ++j)
-    CK(launch_trsm_right<T>(1, R, g.ldr, n, w + (size_t)j * n, 1, 1, 1, h->st));
+  CK(launch_trsv_upper<T>(R, g.ldr, n, w, n, k, h->st));
   const T* z = w;
   // Az, r = y - A x
   CK(launch_gemm_general<T>(0, 0, m, k, n, T(1), A, lda, z, n, T(0), Az, m, h->st));
   CK(launch_axpy2d<T>(m, k, T(1), y, 1, ldy, r, 1, m, true, h->st));
   CK(launch_gemm_general<T>(0, 0, m, k, n, T(-1), A, lda, x, ldx, T(1), r, m, h->st));
   // Abar += r z^T - (A z) x^T;  ybar += A z
-  if (Abar) {
-    CK(launch_gemm_general<T>(0, 1, m, n, k, T(1), r, m, z, n, T(1), Abar, ldab, h->st));
-    CK(launch_gemm_general<T>(0, 1, m, n, k, T(-1), Az, m, x, ldx, T(1), Abar, ldab, h->st));
-  }
+  if (Abar) CK(launch_rank2<T>(m, n, k, r, m, z, n, Az, m, x, ldx, Abar, ldab, h->st));
   if (ybar) CK(launch_axpy2d<T>(m, k, T(1), Az, 1, m, ybar, 1, ldyb, false, h->st));
   return CQR_OK;
 }

@@ -74,6 +74,7 @@ cudaError_t bounds_take_panel_reg(int* code, int* site);
 cudaError_t bounds_take_panel_blk(int* code, int* site);
 cudaError_t bounds_take_lstsq(int* code, int* site);
 cudaError_t bounds_take_f64_gemm(int* code, int* site);
+cudaError_t bounds_take_adjoint(int* code, int* site);
 cudaError_t bounds_take_tc(int* code, int* site);
 // A guarded write past a four-element array (the bounds-checked build's self-test).
 cudaError_t launch_bounds_selftest(int idx, cudaStream_t st);
@@ -216,6 +217,21 @@ cudaError_t launch_axpy2d(int64_t rows, int64_t cols, T alpha, const T* X, int64
 template <typename T>
 cudaError_t launch_trsm_right(int trans, const T* R, int64_t ldr, int64_t n, T* B, int64_t rs,
                               int64_t cs, int64_t m, cudaStream_t st);
+
+// R^T x = b in place for R upper triangular, k right-hand sides.
+template <typename T>
+cudaError_t launch_trsv_upper_t(const T* R, int64_t ldr, int64_t n, T* x, int64_t ldx, int64_t k,
+                                cudaStream_t st);
+// C (M x N) += A B^T - D E^T, k columns.
+template <typename T>
+cudaError_t launch_rank2(int64_t M, int64_t N, int k, const T* A, int64_t lda, const T* B, int64_t ldb,
+                         const T* D, int64_t ldd, const T* E, int64_t lde, T* C, int64_t ldc,
+                         cudaStream_t st);
+// Inverses of the tri_inverse_block()-sized diagonal blocks of R (upper), column-major, one after
+// the other in V.
+int tri_inverse_block();
+template <typename T>
+cudaError_t launch_tri_inverse(const T* R, int64_t ldr, int64_t n, T* V, cudaStream_t st);
 
 // ---------------------------------------------------------------- batches of instances
 // One instance of a batch of independent coded QRs (device copy).  Every batched launch maps
