@@ -677,12 +677,16 @@ __device__ void b_update(BCtx<G>& c, const float* P, int64_t cs, int nr, int bk,
 // In-launch recovery of one instance (a6 + a7) by its cluster, at the start of its erasure
 // panel: the listed tiles are poisoned (NaN), then every code with lost tiles is decoded.  The
 // coefficient tables go in the panel pool, which is free between panels.  Cluster barriers
-// order the poisoning before the decode and the decode before the next panel.
+// order the update before the poisoning, that before the decode and the decode before the next
+// panel.
 template <int G>
 __device__ void b_recover(BCtx<G>& c, const BatchInst<float>& I, const BatchTile* __restrict__ tiles,
                           const BatchPlan* __restrict__ plans, const double* __restrict__ Gt,
                           const double* __restrict__ Gh) {
   const Geo& g = I.g;
+  // every CTA of the cluster writes tiles of all rows: the others have finished the update of
+  // the panel before
+  if (G > 1) cl_sync(); else __syncthreads();
   for (int e = I.tile0; e < I.tile0 + I.ntiles; ++e) {
     const BatchTile t = tiles[e];
     float* X = t.isR ? I.R : I.Q;
