@@ -26,6 +26,7 @@
 #include "cqr_batched.cuh"
 #include "cqr_decode.cuh"
 #include "cqr_device.cuh"
+#include "cqr_subblock.cuh"
 
 namespace cqr {
 
@@ -109,7 +110,6 @@ __device__ __forceinline__ void ph_end() {
 //           panel it is scratch for per-CTA sums
 constexpr int kKT = 64;        // rows per pipeline stage
 constexpr int kLDS = kKT + 4;  // row stride of a staged column (16-byte aligned)
-constexpr int kMaxStages = 8;
 constexpr int kPanelScratch = 8192 + kBW * 2 * kBMax;  // per-CTA sums and warp partials
 
 struct BLayout {
@@ -127,10 +127,6 @@ __host__ __device__ inline BLayout b_layout(int G) {
   return L;
 }
 
-// Floats of one pipeline stage for a panel of width bk: kWC columns of B and bk (rounded up
-// to 4) columns of Qbar, kKT rows each.
-__host__ __device__ inline int stage_floats(int bk) { return (kWC + (bk + 3) / 4 * 4) * kLDS; }
-
 template <int G>
 struct BCtx {
   float* sm;
@@ -145,21 +141,9 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int sr
                : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// Wait until at most n committed groups are pending (n is rounded down to 0 .. 6).
 template <int N>
 __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void cp_wait_dyn(int n) {
-  switch (n) {
-    case 6: cp_wait<6>(); break;
-    case 5: cp_wait<5>(); break;
-    case 4: cp_wait<4>(); break;
-    case 3: cp_wait<3>(); break;
-    case 2: cp_wait<2>(); break;
-    case 1: cp_wait<1>(); break;
-    default: cp_wait<0>(); break;
-  }
 }
 
 // Sum over the cluster of this CTA's values loc[0 .. n) (already summed over the CTA) into
@@ -402,29 +386,39 @@ __device__ __forceinline__ void cta_start_sums(BCtx<G>& c, const float* P, int64
   }
 }
 
-// One panel: columns kb .. kb+bk-1 of the instance, this CTA's rows [0, nr) of the slice at
-// P (column stride cs).  Writes R's diagonal block (rank 0).  Returns false on breakdown.
+// One panel by the column recurrence, from its column jb: columns kb .. kb+bk-1 of the instance,
+// this CTA's rows [0, nr) of the slice at P (column stride cs).  Writes R's diagonal block
+// (rank 0).  jb > 0: columns before jb are done, the later ones updated by them, and eta holds
+// the ICGS thresholds.  Returns false on breakdown.
 template <int G, int RPT>
 __device__ bool b_panel(BCtx<G>& c, float* P, int64_t cs, int nr, int bk, float* R, int64_t ldr,
-                        int kb, double tau2, int* status) {
+                        int kb, double tau2, int* status, int jb) {
   float* v = c.sm + c.L.small;
   float* eta = v + kBMax;
   float* sv = eta + kBMax;
   float* loc = c.sm + c.L.pool;  // per-CTA sums (the pipeline stages are idle during the panel)
   float* tmp = c.sm + c.L.rbar;  // cluster sums
+  const bool icgs = tau2 > 0.0;
+  if (jb > 0) {
+    cta_colsums<G>(c, bk - jb, nr, loc,
+                   [&](int a, int r) { return P[r + (jb + a) * cs] * P[r + jb * cs]; });
+    cluster_sum<G>(c, loc, bk - jb, tmp);
+    for (int a = c.tid; a < bk - jb; a += kBT) v[jb + a] = tmp[a];
+    __syncthreads();
+  } else {
   // step 0: v_a = p_a^T p_0 and eta_a = p_a^T p_a
   cta_start_sums<G, RPT>(c, P, cs, nr, bk, loc);
   cluster_sum<G>(c, loc, 2 * bk, tmp);
   // eta_a is kept as the ICGS threshold: the FP64 product tau^2 eta_a rounded up to FP32, so
   // that the FP32 test v_j < eta_j decides exactly as the FP64 one, with one FP64 product per
   // column instead of one per thread and column
-  const bool icgs = tau2 > 0.0;
   for (int a = c.tid; a < bk; a += kBT) {
     v[a] = tmp[a];
     eta[a] = icgs ? __double2float_ru(tau2 * (double)tmp[bk + a]) : tmp[bk + a];
   }
   __syncthreads();
-  for (int j = 0; j < bk; ++j) {
+  }
+  for (int j = jb; j < bk; ++j) {
     if (j > 0 && icgs && v[j] < eta[j]) {
       // ICGS: project p_j once more on q_0 .. q_{j-1}
       cta_colsums<G>(c, j, nr, loc, [&](int a, int r) { return P[r + a * cs] * P[r + j * cs]; });
@@ -470,208 +464,333 @@ __device__ bool b_panel(BCtx<G>& c, float* P, int64_t cs, int nr, int bk, float*
   return true;
 }
 
-// Trailing update of one panel on this CTA's rows, in chunks of kWC columns:
-//   S = Qbar^T B over this CTA's rows: stages of kKT rows of B and of Qbar stream in through
-//       a cp.async pipeline as deep as the shared-memory pool allows (up to kMaxStages),
-//       two stages per CTA barrier; each thread accumulates a 4 x 4 tile of S over a K-split
-//       share of four-row groups;
-//   Rbar = cluster sum of S (fixed order);  R[kb.., col] = Rbar (rank 0);
-//   B -= Qbar Rbar: the same stages stream in again, each thread updates four rows x two
-//       columns and stores them straight to global memory.
-// Qbar: P (global, rows [0, nr) of the slice, stride cs); B: Qs + col * ldq.
+// The two products of an update, on this CTA's rows [0, nr): with A (na <= kBMax columns at
+// stride as) and B (w <= kWC columns at stride bs) in global memory,
+//   products: rbar[a * kWC + j] = a_a^T b_j over all rows of the cluster,
+//   apply:    b_j <- [j >= keep] b_j - sum_a a_a rbar[a * kWC + j].
+// Rows stream in by cp.async in supers of `spb` stages of kKT rows (as many as half the pool
+// holds), two supers in turn.  A and B may overlap: a super is in shared memory before its rows
+// are written.  Bound by shared-memory reads: a thread forms 8 x 4 sums (12 reads of 16 bytes
+// per 128 products; 4 x 4 and 4 x 2 tiles before took 16 and 24), and the copies' addresses are
+// formed once per product, not per stage.
+template <int G>
+struct BStream {
+  static constexpr int kCopies = (kWC + kBMax) * (kKT / 4) / kBT;  // 16-byte pieces per thread and stage
+  BCtx<G>& c;
+  int nr, ncb, nca, sf, spb, nsup;
+  const float* src[kCopies];
+  uint32_t dst[kCopies];
+  bool ok[kCopies];
+  int q4;
+  float* pool;
+
+  // ncb, nca: staged columns of B and A (zero-filled past w and na)
+  __device__ BStream(BCtx<G>& c_, const float* A, int64_t as, int na, int nca_, const float* B,
+                     int64_t bs, int w, int ncb_, int nr_, int pool_floats)
+      : c(c_), nr(nr_), ncb(ncb_), nca(nca_), pool(c_.sm + c_.L.pool) {
+    sf = (ncb + nca) * kLDS;
+    const int nst = pool_floats / sf;
+    spb = nst / 2 < 8 ? nst / 2 : 8;
+    nsup = (nr + spb * kKT - 1) / (spb * kKT);
+    q4 = c.tid % (kKT / 4);
+#pragma unroll
+    for (int u = 0; u < kCopies; ++u) {
+      const int j = c.tid / (kKT / 4) + u * (kBT / (kKT / 4));
+      const bool isB = j < ncb;
+      const int col = isB ? j : j - ncb;
+      ok[u] = isB ? col < w : col < na;
+      src[u] = (isB ? B + (ok[u] ? col : 0) * bs : A + (ok[u] ? col : 0) * as) + 4 * q4;
+      dst[u] = j < ncb + nca ? s_addr(pool) + 4u * (uint32_t)(j * kLDS + 4 * q4) : 0u;
+    }
+  }
+  __device__ void issue(int s) {
+    if (s < nsup)
+      for (int t = 0; t < spb; ++t) {
+        const int r0 = (s * spb + t) * kKT, r = r0 + 4 * q4;
+        if (r0 >= nr) break;
+        const uint32_t off = 4u * (uint32_t)(((s & 1) * spb + t) * sf);
+        const int left = nr - r;
+        const int nb = left >= 4 ? 16 : left > 0 ? 4 * left : 0;
+#pragma unroll
+        for (int u = 0; u < kCopies; ++u)
+          if (dst[u]) cp_async16(dst[u] + off, src[u] + (nb ? r0 : -4 * q4), ok[u] ? nb : 0);
+      }
+    cp_commit();
+  }
+  __device__ const float* stage(int s, int t) const { return pool + ((s & 1) * spb + t) * sf; }
+};
+
+template <int G>
+__device__ void b_products(BCtx<G>& c, const float* A, int64_t as, int na, const float* B, int64_t bs,
+                           int w, int nr, int pool_floats) {
+  const int nj = (w + 3) / 4, na8 = (na + 7) / 8;
+  const int tiles = na8 * nj;
+  int ks_n = kBT / tiles;
+  const int fit = pool_floats / (8 * na8 * kWC);
+  ks_n = ks_n < 16 ? ks_n : 16;
+  ks_n = ks_n < fit ? ks_n : fit;
+  const int t_id = c.tid % tiles, ks = c.tid / tiles;
+  const bool active = ks < ks_n;
+  // columns ai + x na8 of A and ji + y nj of B: neighbouring lanes read neighbouring staged
+  // columns, so the 16-byte reads do not conflict
+  const int ai = t_id % na8, ji = t_id / na8;
+  BStream<G> st(c, A, as, na, 8 * na8, B, bs, w, 4 * nj, nr, pool_floats);
+  float acc[8][4];
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
+  __syncthreads();  // the previous readers of the pool are done
+  st.issue(0);
+  st.issue(1);
+  for (int s = 0; s < st.nsup; ++s) {
+    ph_mark(PH_SPROD);
+    cp_wait<1>();
+    __syncthreads();
+    ph_mark(PH_SPROD_WAIT);
+    if (active) {
+      const int rows = nr - s * st.spb * kKT;
+      const int ng = ((rows < st.spb * kKT ? rows : st.spb * kKT) + 3) / 4;
+      for (int g = ks; g < ng; g += ks_n) {
+        const float* Bt = st.stage(s, g / (kKT / 4)) + 4 * (g % (kKT / 4));
+        const float* At = Bt + st.ncb * kLDS;
+        float4 bv[4];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) bv[y] = *reinterpret_cast<const float4*>(Bt + (ji + y * nj) * kLDS);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          const float4 q = *reinterpret_cast<const float4*>(At + (ai + x * na8) * kLDS);
+#pragma unroll
+          for (int y = 0; y < 4; ++y)
+            acc[x][y] = fmaf(q.w, bv[y].w, fmaf(q.z, bv[y].z, fmaf(q.y, bv[y].y, fmaf(q.x, bv[y].x, acc[x][y]))));
+        }
+      }
+    }
+    __syncthreads();
+    st.issue(s + 2);
+  }
+  cp_wait<0>();
+  __syncthreads();
+  ph_mark(PH_SPROD);
+  // K-split partials -> pool[ks][a][j], then a fixed-order sum
+  float* spart = st.pool;
+  float* rbar = c.sm + c.L.rbar;
+  const int ps = 8 * na8 * kWC;
+  if (active)
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) spart[ks * ps + (ai + x * na8) * kWC + ji + y * nj] = acc[x][y];
+  __syncthreads();
+  float* mine = G == 1 ? rbar : c.sm + c.L.cpart + (c.step & 1) * (kBMax * kWC);
+  for (int e = c.tid; e < na * kWC; e += kBT) {
+    float sum = 0.f;
+    if (e % kWC < w)
+      for (int q = 0; q < ks_n; ++q) sum += spart[q * ps + e];
+    mine[e] = sum;
+  }
+  if (G == 1) {
+    __syncthreads();
+    return;
+  }
+  cl_sync();
+  const uint32_t base = s_addr(mine);
+  for (int e = c.tid; e < na * kWC; e += kBT) {
+    float sum = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) sum += ld_cl(base + 4u * (uint32_t)e, (uint32_t)g);
+    rbar[e] = sum;
+  }
+  ++c.step;
+  __syncthreads();
+}
+
+// After a CTA barrier behind the last write of rbar.
+template <int G>
+__device__ void b_apply(BCtx<G>& c, const float* A, int64_t as, int na, float* B, int64_t bs, int w,
+                        int keep, int nr, int pool_floats) {
+  const float* rbar = c.sm + c.L.rbar;
+  const int nj = (w + 3) / 4;
+  BStream<G> st(c, A, as, na, (na + 3) / 4 * 4, B, bs, w, 4 * nj, nr, pool_floats);
+  // a thread's tile: rows 4 rq .. +3 and 32 + 4 rq .. +3 of a stage, columns 4 cq .. +3; groups of
+  // tps threads take the stages of a super in turn
+  int ncg = 1;
+  while (ncg < nj) ncg *= 2;
+  const int tps = 8 * ncg, ngrp = kBT / tps, grp = c.tid / tps;
+  const int rq = c.tid & 7, cq = (c.tid % tps) >> 3;
+  __syncthreads();
+  st.issue(0);
+  st.issue(1);
+  for (int s = 0; s < st.nsup; ++s) {
+    ph_mark(PH_UPDATE);
+    cp_wait<1>();
+    __syncthreads();
+    ph_mark(PH_UPDATE_WAIT);
+    if (cq < nj)
+      for (int t = grp; t < st.spb; t += ngrp) {
+        const int r0 = (s * st.spb + t) * kKT;
+        if (r0 >= nr) break;
+        const float* Bt = st.stage(s, t);
+        const float* At = Bt + st.ncb * kLDS + 4 * rq;
+        float o[8][4];
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) o[x][y] = 0.f;
+#pragma unroll 4
+        for (int a = 0; a < na; ++a) {
+          const float4 q0 = *reinterpret_cast<const float4*>(At + a * kLDS);
+          const float4 q1 = *reinterpret_cast<const float4*>(At + a * kLDS + 32);
+          const float4 rv = *reinterpret_cast<const float4*>(rbar + a * kWC + 4 * cq);
+          const float qs[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+          const float rs[4] = {rv.x, rv.y, rv.z, rv.w};
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) o[x][y] = fmaf(qs[x], rs[y], o[x][y]);
+        }
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          const int j = 4 * cq + y;
+          if (j >= w) break;
+          const bool add = j >= keep;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int r = r0 + 4 * rq + 32 * h;
+            if (r >= nr) continue;
+            float4 b4 = *reinterpret_cast<const float4*>(Bt + j * kLDS + 4 * rq + 32 * h);
+            if (!add) b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float v[4] = {b4.x - o[4 * h][y], b4.y - o[4 * h + 1][y], b4.z - o[4 * h + 2][y],
+                                b4.w - o[4 * h + 3][y]};
+            float* dst = B + r + (int64_t)j * bs;
+            if (r + 4 <= nr) {
+              *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+#pragma unroll
+              for (int x = 0; x < 4; ++x)
+                if (r + x < nr) dst[x] = v[x];
+            }
+          }
+        }
+      }
+    __syncthreads();
+    st.issue(s + 2);
+  }
+  cp_wait<0>();
+  __syncthreads();
+  ph_mark(PH_UPDATE);
+}
+
+// Trailing update of one panel on this CTA's rows, in chunks of kWC columns: Rbar = Qbar^T B,
+// R[kb.., col] = Rbar (rank 0), B -= Qbar Rbar.  Qbar: P (rows [0, nr) of the slice, stride cs);
+// B: Qs + col * ldq.
 template <int G>
 __device__ void b_update(BCtx<G>& c, const float* P, int64_t cs, int nr, int bk, float* Qs,
                          int64_t ldq, int64_t col_begin, int64_t col_end, float* R, int64_t ldr,
                          int kb, int pool_floats) {
-  float* pool = c.sm + c.L.pool;
-  float* spart = pool;             // K-split partials after the K loop
-  float* rbar = c.sm + c.L.rbar;   // [bk][kWC]
-  const int sf = stage_floats(bk);
-  int nst = pool_floats / sf;
-  if (nst > kMaxStages) nst = kMaxStages;
-  // two stages per CTA barrier when at least four fit (one otherwise); `depth` stages are in
-  // flight ahead of the ones being consumed
-  const int spb = nst >= 4 ? 2 : 1;
-  const int depth = nst - spb;
-  const int bkq = (bk + 3) / 4;
-  const int tiles = bkq * (kWC / 4);
-  int ks_n = kBT / tiles;
-  if (ks_n > 8) ks_n = 8;
-  if (ks_n < 1) ks_n = 1;
-  const int t_id = c.tid % tiles, ks = c.tid / tiles;
-  const bool active = c.tid < tiles * ks_n;
-  // a thread's S tile: columns ai + x bkq of Qbar and ji + 16 y of B (x, y < 4); neighbouring
-  // lanes read neighbouring staged columns, so the 16-byte shared loads do not conflict
-  const int ai = t_id % bkq, ji = t_id / bkq;
-  const int nkt = (nr + kKT - 1) / kKT;
-  const uint32_t pool_u = s_addr(pool);
-  // GEMM2 thread layout: rows 4*rq4 .. +3 of a stage, columns 2*cp, 2*cp+1
-  const int rq4 = c.tid % (kKT / 4), cp = c.tid / (kKT / 4);
+  const float* rbar = c.sm + c.L.rbar;
   for (int64_t c0 = col_begin; c0 < col_end; c0 += kWC) {
     const int wc = (int)((col_end - c0) < kWC ? (col_end - c0) : kWC);
-    // stage t: B rows [r0, r0 + kKT) x columns [c0, c0 + kWC), then Qbar rows [r0, r0 + kKT) x
-    // columns [0, bk), as 16-byte pieces (four rows of one column); rows >= nr and columns
-    // beyond the block are zero-filled.  One commit group per stage (empty past the end).
-    auto issue = [&](int t) {
-      if (t < nkt) {
-        const uint32_t base = pool_u + 4u * (uint32_t)((t % nst) * sf);
-        const int r0 = t * kKT;
-        for (int e = c.tid; e < (kWC + bkq * 4) * (kKT / 4); e += kBT) {
-          const int q4 = e % (kKT / 4), j = e / (kKT / 4);
-          const int r = r0 + 4 * q4;
-          const bool isB = j < kWC;
-          const int col = isB ? j : j - kWC;
-          const bool ok = (isB ? col < wc : col < bk) && r < nr;
-          const int nb = ok ? ((nr - r) >= 4 ? 16 : 4 * (nr - r)) : 0;
-          const float* src = isB ? Qs + (ok ? r : 0) + (c0 + (ok ? col : 0)) * ldq
-                                 : P + (ok ? r : 0) + (ok ? col : 0) * cs;
-          cp_async16(base + 4u * (uint32_t)(j * kLDS + 4 * q4), src, nb);
-        }
-      }
-      cp_commit();
-    };
-    auto stage = [&](int t) { return pool + (t % nst) * sf; };
-    // ---------------------------------------------------------------- S = Qbar^T B
-    float acc[4][4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-    __syncthreads();  // the previous readers of the pool are done
-    // one stage of S: this thread's 4 x 4 tile over its K-split share of the four-row groups
-    auto s_stage = [&](int t) {
-      const int r0 = t * kKT;
-      const int kr = (nr - r0) < kKT ? (nr - r0) : kKT;
-      const int ng = (kr + 3) / 4;
-      if (active) {
-        const float* Bt = stage(t);
-        const float* At = Bt + kWC * kLDS;
-        for (int g4 = ks; g4 < ng; g4 += ks_n) {
-          const int rr = 4 * g4;
-          float4 qv[4], bv[4];
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-            qv[x] = (ai + x * bkq < bk) ? *reinterpret_cast<const float4*>(At + (ai + x * bkq) * kLDS + rr)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int y = 0; y < 4; ++y)
-            bv[y] = *reinterpret_cast<const float4*>(Bt + (ji + 16 * y) * kLDS + rr);
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-              float a = acc[x][y];
-              a = fmaf(qv[x].x, bv[y].x, a);
-              a = fmaf(qv[x].y, bv[y].y, a);
-              a = fmaf(qv[x].z, bv[y].z, a);
-              a = fmaf(qv[x].w, bv[y].w, a);
-              acc[x][y] = a;
-            }
-        }
-      }
-    };
-    for (int t = 0; t < depth; ++t) issue(t);
-    for (int t = 0; t < nkt; t += spb) {
-      ph_mark(PH_SPROD);
-      cp_wait_dyn(depth - spb);
-      __syncthreads();
-      ph_mark(PH_SPROD_WAIT);
-      for (int u = 0; u < spb; ++u) issue(t + depth + u);
-      for (int u = 0; u < spb; ++u)
-        if (t + u < nkt) s_stage(t + u);
-    }
-    cp_wait<0>();
-    __syncthreads();
-    ph_mark(PH_SPROD);
-    // K-split partials -> spart[ks][a][j] (ld kWC), then a fixed-order sum
-    if (active)
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y)
-          if (ai + x * bkq < bk) spart[ks * (bkq * 4 * kWC) + (ai + x * bkq) * kWC + ji + 16 * y] = acc[x][y];
-    __syncthreads();
-    if (G == 1) {
-      for (int e = c.tid; e < bk * kWC; e += kBT) {
-        float sum = 0.f;
-        for (int q = 0; q < ks_n; ++q) sum += spart[q * (bkq * 4 * kWC) + e];
-        rbar[e] = sum;
-      }
-      __syncthreads();
-    } else {
-      float* mine = c.sm + c.L.cpart + (c.step & 1) * (kBMax * kWC);
-      for (int e = c.tid; e < bk * kWC; e += kBT) {
-        float sum = 0.f;
-        for (int q = 0; q < ks_n; ++q) sum += spart[q * (bkq * 4 * kWC) + e];
-        mine[e] = sum;
-      }
-      cl_sync();
-      const uint32_t base = s_addr(mine);
-      for (int e = c.tid; e < bk * kWC; e += kBT) {
-        float sum = 0.f;
-#pragma unroll
-        for (int g = 0; g < G; ++g) sum += ld_cl(base + 4u * (uint32_t)e, (uint32_t)g);
-        rbar[e] = sum;
-      }
-      ++c.step;
-      __syncthreads();
-    }
+    b_products<G>(c, P, cs, bk, Qs + c0 * ldq, ldq, wc, nr, pool_floats);
     if (c.rank == 0)
       for (int e = c.tid; e < bk * wc; e += kBT) {
         const int a = e / wc, j = e % wc;
         R[(kb + a) + (c0 + j) * ldr] = rbar[a * kWC + j];
       }
     ph_mark(PH_RBAR);
-    // ---------------------------------------------------------------- B -= Qbar Rbar
-    // one stage of the update: four rows x two columns of B per thread, stored to global
-    auto u_stage = [&](int t) {
-      const int r = t * kKT + 4 * rq4;
-      const int j = 2 * cp;
-      if (r < nr && j < wc) {
-        const float* Bt = stage(t);
-        const float* At = Bt + kWC * kLDS;
-        float o[4][2];
+    b_apply<G>(c, P, cs, bk, Qs + c0 * ldq, ldq, wc, 0, nr, pool_floats);
+  }
+}
+
+// One panel in sub-blocks of 16 columns (the arithmetic of cqr_panel_blk.cu): W = P_S^T P[:, j:],
+// Cholesky of its leading block, and one pass that turns P_S into Q_S = P_S U^{-1} and takes
+// Q_S R off the columns behind (P_S (U^{-1} R), with the coefficients of both in rbar).  The
+// slice stays in global memory (L2) and streams through shared memory twice per sub-block
+// instead of once per column.  Returns the columns done: up to the first that fails the ICGS
+// test, has no fine pivot or would lose digits; the column recurrence takes over there.
+template <int G>
+__device__ int b_panel_blocks(BCtx<G>& c, float* P, int64_t cs, int nr, int bk, float* R, int64_t ldr,
+                              int kb, double tau2, int pool_floats) {
+  constexpr int S = kS<float>;
+  __shared__ __align__(16) float sU[S * S], sLi[S * S], sRow[16 * S], sD[S];
+  __shared__ float sNrm[S];
+  __shared__ int sGood;
+  float* eta = c.sm + c.L.small + kBMax;
+  float* loc = c.sm + c.L.pool;
+  float* rbar = c.sm + c.L.rbar;
+  const bool icgs = tau2 > 0.0;
+  for (int e = c.tid; e < 16 * S; e += kBT) sRow[e] = 0.f;
+  if (icgs) {
+    cta_colsums<G>(c, bk, nr, loc, [&](int a, int r) { return P[r + a * cs] * P[r + a * cs]; });
+    cluster_sum<G>(c, loc, bk, rbar);
+    for (int a = c.tid; a < bk; a += kBT) eta[a] = __double2float_ru(tau2 * (double)rbar[a]);
+    __syncthreads();
+  }
+  int j = 0;
+  while (j < bk) {
+    const int w = bk - j, n = w < S ? w : S;
+    float* Pj = P + (int64_t)j * cs;
+    b_products<G>(c, Pj, cs, n, Pj, cs, w, nr, pool_floats);
+    if (c.warp == 0) {
+      if (c.lane < n) sNrm[c.lane] = sqrtf(rbar[c.lane * kWC + c.lane]);
+      int gd = cholesky<float>(rbar, kWC, n, sU, sLi, sD, sRow);
+      float amp = 0.f;
+      if (c.lane < gd)
+#pragma unroll 4
+        for (int k = 0; k < S; ++k) amp += fabsf(sLi[c.lane * S + k]) * sNrm[k < n ? k : n - 1];
+      const unsigned bad = __ballot_sync(0xffffffffu, c.lane > 0 && c.lane < gd && !(amp <= kMaxAmp));
+      if (bad) gd = min(gd, __ffs(bad) - 1);
+      const bool test = icgs && c.lane < gd && j + c.lane > 0;
+      const unsigned f = __ballot_sync(0xffffffffu, test && sD[test ? c.lane : 0] < eta[test ? j + c.lane : 0]);
+      if (f) gd = min(gd, __ffs(f) - 1);
+      if (c.lane == 0) sGood = gd;
+    }
+    __syncthreads();
+    const int good = sGood;
+    if (good == 0) return j;
+    // column jj: its rows of R, and in rbar the coefficients a_k of -sum_k p_k a_k: -U^{-1} for the
+    // sub-block's own columns, U^{-1} R behind them
+    for (int jj = c.tid; jj < w; jj += kBT) {
+      float r[S];
+      if (jj < good) {
 #pragma unroll
-        for (int x = 0; x < 4; ++x) o[x][0] = o[x][1] = 0.f;
-        for (int a = 0; a < bk; ++a) {
-          const float4 q = *reinterpret_cast<const float4*>(At + a * kLDS + 4 * rq4);
-          const float2 rv = *reinterpret_cast<const float2*>(rbar + a * kWC + j);
-          o[0][0] = fmaf(q.x, rv.x, o[0][0]); o[0][1] = fmaf(q.x, rv.y, o[0][1]);
-          o[1][0] = fmaf(q.y, rv.x, o[1][0]); o[1][1] = fmaf(q.y, rv.y, o[1][1]);
-          o[2][0] = fmaf(q.z, rv.x, o[2][0]); o[2][1] = fmaf(q.z, rv.y, o[2][1]);
-          o[3][0] = fmaf(q.w, rv.x, o[3][0]); o[3][1] = fmaf(q.w, rv.y, o[3][1]);
-        }
+        for (int a = 0; a < S; ++a) r[a] = a <= jj ? sU[a * S + jj] : 0.f;
+      } else {
+        float x[S];
 #pragma unroll
-        for (int y = 0; y < 2; ++y) {
-          if (j + y >= wc) break;
-          const float4 b4 = *reinterpret_cast<const float4*>(Bt + (j + y) * kLDS + 4 * rq4);
-          float* dst = Qs + r + (c0 + j + y) * ldq;
-          if (r + 4 <= nr) {
-            *reinterpret_cast<float4*>(dst) =
-                make_float4(b4.x - o[0][y], b4.y - o[1][y], b4.z - o[2][y], b4.w - o[3][y]);
-          } else {
-            const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
+        for (int a = 0; a < S; ++a) x[a] = a < good ? rbar[a * kWC + jj] : 0.f;
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
-              if (r + x < nr) dst[x] = bb[x] - o[x][y];
-          }
+        for (int a = 0; a < S; ++a) {
+          float t = 0.f;
+          if (a < good)
+#pragma unroll
+            for (int m = 0; m <= a; ++m) t = fmaf(sLi[a * S + m], x[m], t);
+          r[a] = t;
         }
       }
-    };
-    for (int t = 0; t < depth; ++t) issue(t);
-    for (int t = 0; t < nkt; t += spb) {
-      ph_mark(PH_UPDATE);
-      cp_wait_dyn(depth - spb);
-      __syncthreads();
-      ph_mark(PH_UPDATE_WAIT);
-      for (int u = 0; u < spb; ++u) issue(t + depth + u);
-      for (int u = 0; u < spb; ++u)
-        if (t + u < nkt) u_stage(t + u);
+      if (c.rank == 0)
+        for (int a = 0; a < good && a <= jj; ++a)
+          R[(kb + j + a) + (int64_t)(kb + j + jj) * ldr] = r[a];
+#pragma unroll
+      for (int k = 0; k < S; ++k) {
+        if (k >= good) break;
+        float t = 0.f;
+        if (jj < good) {
+          t = k <= jj ? -sLi[jj * S + k] : 0.f;
+        } else {
+#pragma unroll
+          for (int a = k; a < S; ++a)
+            if (a < good) t = fmaf(sLi[a * S + k], r[a], t);
+        }
+        rbar[k * kWC + jj] = t;
+      }
     }
-    cp_wait<0>();
-    ph_mark(PH_UPDATE);
+    __syncthreads();
+    b_apply<G>(c, Pj, cs, good, Pj, cs, w, good, nr, pool_floats);
+    j += good;
+    if (good < n) return j;
   }
-  __syncthreads();
+  return bk;
 }
 
 // In-launch recovery of one instance (a6 + a7) by its cluster, at the start of its erasure
@@ -763,33 +882,37 @@ __global__ void __launch_bounds__(kBT, 1) k_b_factor(BatchInst<float>* __restric
       }
       const int kb = k * I.b;
       const int bk = (int)std::min<int64_t>(I.b, g.n - kb);
-      // ICGS on the panel slice: in the shared-memory pool (after the panel's scratch) when it
-      // fits, else in place in global memory (L2); the update then streams it from global
       float* Pg = Qs + (int64_t)kb * g.ldq;
-      const int rpad = (nr + 3) / 4 * 4;
-      const bool in_smem = rpad * bk <= panel_cap - kPanelScratch;
-      float* P = in_smem ? smem + c.L.pool + kPanelScratch : Pg;
-      const int64_t cs = in_smem ? rpad : g.ldq;
-      if (in_smem) {
-        for (int e = c.tid; e < rpad * bk; e += kBT) {
-          const int r = e % rpad, a = e / rpad;
-          P[e] = (r < nr) ? Pg[r + (int64_t)a * g.ldq] : 0.f;
+      const int done = b_panel_blocks<G>(c, Pg, g.ldq, nr, bk, I.R, g.ldr, kb, tau2, panel_cap);
+      if (done < bk) {
+        // the column recurrence on the slice: in the shared-memory pool (after the panel's
+        // scratch) when it fits, else in place in global memory (L2)
+        const int rpad = (nr + 3) / 4 * 4;
+        const bool in_smem = rpad * bk <= panel_cap - kPanelScratch;
+        float* P = in_smem ? smem + c.L.pool + kPanelScratch : Pg;
+        const int64_t cs = in_smem ? rpad : g.ldq;
+        __syncthreads();
+        if (in_smem) {
+          for (int e = c.tid; e < rpad * bk; e += kBT) {
+            const int r = e % rpad, a = e / rpad;
+            P[e] = (r < nr) ? Pg[r + (int64_t)a * g.ldq] : 0.f;
+          }
+          __syncthreads();
         }
+        if (nr <= 4 * kBT)
+          ok = b_panel<G, 4>(c, P, cs, nr, bk, I.R, g.ldr, kb, tau2, I.status, done);
+        else if (nr <= 8 * kBT)
+          ok = b_panel<G, 8>(c, P, cs, nr, bk, I.R, g.ldr, kb, tau2, I.status, done);
+        else
+          ok = b_panel<G, 10>(c, P, cs, nr, bk, I.R, g.ldr, kb, tau2, I.status, done);
+        if (!ok) break;
+        if (in_smem)
+          for (int e = c.tid; e < rpad * bk; e += kBT) {
+            const int r = e % rpad, a = e / rpad;
+            if (r < nr) Pg[r + (int64_t)a * g.ldq] = P[e];
+          }
         __syncthreads();
       }
-      if (nr <= 4 * kBT)
-        ok = b_panel<G, 4>(c, P, cs, nr, bk, I.R, g.ldr, kb, tau2, I.status);
-      else if (nr <= 8 * kBT)
-        ok = b_panel<G, 8>(c, P, cs, nr, bk, I.R, g.ldr, kb, tau2, I.status);
-      else
-        ok = b_panel<G, 10>(c, P, cs, nr, bk, I.R, g.ldr, kb, tau2, I.status);
-      if (!ok) break;
-      if (in_smem)
-        for (int e = c.tid; e < rpad * bk; e += kBT) {
-          const int r = e % rpad, a = e / rpad;
-          if (r < nr) Pg[r + (int64_t)a * g.ldq] = P[e];
-        }
-      __syncthreads();
       ph_mark(PH_PANEL);
       b_update<G>(c, Pg, g.ldq, nr, bk, Qs, g.ldq, kb + bk, g.N, I.R, g.ldr, kb, panel_cap);
     }
@@ -852,7 +975,7 @@ int max_clusters_g(int panel_cap) {
 int b_recover_floats() { return (int)((sizeof(DecodeScratch<float>) + sizeof(float) - 1) / sizeof(float)) + 4; }
 
 int b_panel_cap_floats(int G) {
-  const size_t cap = 227 * 1024 / sizeof(float) - 64;  // static shared and alignment slack
+  const size_t cap = 227 * 1024 / sizeof(float) - 1024;  // static shared memory (4 KB at most)
   return (int)(cap - (size_t)b_layout(G).total);
 }
 
