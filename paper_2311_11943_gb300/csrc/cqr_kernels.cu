@@ -37,31 +37,55 @@ __device__ double draw_value(uint64_t& s, int gdist) {
   return sqrt(-2.0 * log(u1)) * cos(6.283185307179586476925286766559 * u2);  // Box-Muller
 }
 
+// SplitMix64's state is its seed plus a multiple of a constant, so draw k needs no earlier draw:
+// every thread forms its own values.  A zero draw (probability 2^-53) is skipped by the stream and
+// shifts all later ones: then one thread draws them in turn.  f = 4, p = 16: 40 -> 7 us, the draws'
+// FP64 arithmetic on one lane before, the launch now.
 template <typename T>
-__global__ void k_generator(int f, int p_r, int p_c, uint64_t seed, int gdist, double* Gt,
-                            double* Gh, T* Gt_t, T* Gh_t) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  uint64_t s = seed;
-  const int nv = p_r - f;
-  for (int i = 0; i < f; ++i)
-    for (int t = 0; t < nv; ++t) Gt[i * p_r + f + t] = draw_value(s, gdist);
-  for (int i = 0; i < f; ++i)
-    for (int l = 0; l < f; ++l) {
-      double acc = 0.0;
-      for (int t = 0; t < nv; ++t)
-        acc = __dadd_rn(acc, __dmul_rn(Gt[i * p_r + f + t], Gt[l * p_r + f + t]));
-      Gt[i * p_r + l] = __dmul_rn(-0.5, acc);
+__global__ void __launch_bounds__(256) k_generator(int f, int p_r, int p_c, uint64_t seed, int gdist,
+                                                   double* Gt, double* Gh, T* Gt_t, T* Gh_t) {
+  const int nv = p_r - f, tid = threadIdx.x;
+  const int count = f * nv + p_c * f, per = gdist == 0 ? 1 : 2;  // values, draws per value
+  // value i of the stream: V~ row-major, then G~_h row-major
+  auto put = [&](int i, double v) {
+    if (i < f * nv) {
+      const int e = (i / nv) * p_r + f + i % nv;
+      Gt[e] = v;
+      Gt_t[e] = (T)v;
+    } else {
+      Gh[i - f * nv] = v;
+      Gh_t[i - f * nv] = (T)v;
     }
-  for (int j = 0; j < p_c; ++j)
-    for (int l = 0; l < f; ++l) Gh[j * f + l] = draw_value(s, gdist);
-  for (int e = 0; e < f * p_r; ++e) Gt_t[e] = (T)Gt[e];
-  for (int e = 0; e < f * p_c; ++e) Gh_t[e] = (T)Gh[e];
+  };
+  int zero = 0;
+  for (int i = tid; i < count; i += 256) {
+    uint64_t s = seed + (uint64_t)(i * per) * 0x9E3779B97F4A7C15ULL;
+    for (int k = 0; k < per; ++k) {
+      uint64_t t = s + (uint64_t)k * 0x9E3779B97F4A7C15ULL;
+      zero |= (splitmix64_next(t) >> 11) == 0;
+    }
+    put(i, draw_value(s, gdist));
+  }
+  if (__syncthreads_or(zero) && tid == 0) {
+    uint64_t s = seed;
+    for (int i = 0; i < count; ++i) put(i, draw_value(s, gdist));
+  }
+  __syncthreads();
+  for (int e = tid; e < f * f; e += 256) {
+    const int i = e / f, l = e % f;
+    double acc = 0.0;
+    for (int t = 0; t < nv; ++t)
+      acc = __dadd_rn(acc, __dmul_rn(Gt[i * p_r + f + t], Gt[l * p_r + f + t]));
+    const double v = __dmul_rn(-0.5, acc);
+    Gt[i * p_r + l] = v;
+    Gt_t[i * p_r + l] = (T)v;
+  }
 }
 
 template <typename T>
 cudaError_t launch_generator(int f, int p_r, int p_c, uint64_t seed, int gdist, double* Gt,
                              double* Gh, T* Gt_t, T* Gh_t, cudaStream_t st) {
-  k_generator<T><<<1, 32, 0, st>>>(f, p_r, p_c, seed, gdist, Gt, Gh, Gt_t, Gh_t);
+  k_generator<T><<<1, 256, 0, st>>>(f, p_r, p_c, seed, gdist, Gt, Gh, Gt_t, Gh_t);
   return cudaGetLastError();
 }
 
