@@ -594,7 +594,7 @@ cqr_status panel_step(cqr_handle h, int t) {
   if (h->tc) {
     {
       ProfScope ps(h, K_TC_SPLIT, 1);
-      CK(tc_split_panel(h->tc, kb, bk, true, buf, h->st));
+      CK(tc_split_panel(h->tc, kb, bk, buf, h->st));
     }
     return tc_update_cols(h, kb, bk, j0, w, buf, 0, 0, h->st);
   }
@@ -688,7 +688,7 @@ cqr_status factor_lookahead(cqr_handle h, int t0, int t1) {
     if (j0 >= g.N) continue;
     {
       ProfScope ps(h, K_TC_SPLIT, 1, A);
-      CK(tc_split_panel(h->tc, kb, bk, true, buf, A));
+      CK(tc_split_panel(h->tc, kb, bk, buf, A));
     }
     const int64_t wn = j0 < g.n ? std::min<int64_t>(g.b, g.n - j0) : g.N - j0;
     if (w_pending) {
@@ -996,6 +996,10 @@ cqr_status coded_qr_factor(cqr_handle h, int32_t t0, int32_t t1) {
   if (h->state == ST_CREATED || h->pending || h->postorth_inplace) return CQR_ESTATE;
   if (t1 < 0) t1 = h->g.panels;
   if (t0 != h->next_panel || t1 < t0 || t1 > h->g.panels) return CQR_ESTATE;
+  if (h->tc && t0 == 0 && t1 > 0) {
+    ProfScope ps(h, K_TC_SPLIT, 1);
+    CK(tc_begin(h->tc, h->st));
+  }
   if (t1 > t0 && h->esz == 4 && lookahead_eligible(h)) {
     cqr_status s = factor_lookahead(h, t0, t1);
     if (s != CQR_OK) return s;

@@ -4,27 +4,40 @@
 // (Appendix A, Algorithm PBMGS, the All-reduce product and the trailing update.)
 //
 // One persistent, warp-specialised kernel computes D = sum_p A_p B_p^T for up to three
-// (A_p, B_p) operand pairs, every operand K-major, with tcgen05.mma kind::tf32 (M = 128,
-// N = 128, K = 8 per instruction) accumulating in tensor memory (TMEM, FP32):
+// (A_p, B_p) operand pairs, every operand K-major, with tcgen05.mma kind::tf32 or kind::f16
+// (M = 128, N = 128, 32 bytes of K per instruction) accumulating in tensor memory (TMEM, FP32):
 //   warp 0      TMA producer: cp.async.bulk.tensor tiles (128-byte swizzle) into a ring of
 //               shared-memory stages, completion counted on an mbarrier per stage
 //   warp 1      allocates TMEM; one thread issues the MMAs and tcgen05.commit's each stage
 //               back to the producer and each finished tile to the epilogue
-//   warps 2-3   3xTF32 only: split the streamed B tile in shared memory into hi = rna_tf32(x)
-//               (in place) and lo = x - hi (second buffer)
+//   warps 2-3   (and 12-13) split the streamed FP32 B tile in shared memory into its hi tile (in
+//               place) and lo tile (the buffer behind it)
 //   warps 4-11  epilogue, two warps per quarter of the TMEM lanes: tcgen05.ld 32 lanes x 32
 //               columns per warp (alternate column chunks), then either store the FP32
 //               partial (GEMM1) or subtract it from Q in place (GEMM2)
 // A work unit is one 128 x 128 output tile, or, for GEMM1 in 3xTF32 with a 256-column panel,
 // the two vertically adjacent tiles of one B tile (two accumulators; B is loaded and split
 // once for both).
-// 3xTF32 (hi*hi + hi*lo + lo*hi) recovers about FP32 accuracy from TF32 products.  The small
-// operands (panel and Rbar) are split into hi/lo planes in global memory by helper kernels.
+// The mode CQR_MMA_3XTF32 forms hi*hi + hi*lo + lo*hi of operands split into two 11-bit halves
+// and so recovers about FP32 accuracy.  The halves are FP16, which has TF32's 11 bits in half the
+// bytes and at twice the rate; what FP16 lacks, TF32's exponent range, comes from a power of two
+// per column (exact to apply and to take out): orthonormal columns are multiplied by 2^12,
+// trailing columns by the power that took their norm into [2^9, 2^10) before the first panel
+// (norms only fall as panels are taken out of a column), the columns of a panel by that of their
+// norm when its block pass begins.  Beyond the halves' 22 bits a split is then off by at most
+// 2^-34 of the column's norm per entry, 2^-10 of the FP32 rounding of the column itself.  Measured
+// against 64 bits: R of 8192 x 8192 1.4e-5 -> 7.7e-6, of 16384 x 2048 6.9e-6 -> 3.7e-6 relative to
+// TF32 halves (fewer roundings in the accumulators).  8192 x 8192, p = 16, b = 256, all panels:
+// Rbar 5.0 -> 2.95 ms, block pass 8.1 -> 5.4 ms, update 4.94 -> 4.38 ms (one pass over the
+// trailing columns, 1.6 ms at the copy rate; bound by the reads of C in the epilogue).
+// The small operands (panel and Rbar) are split into hi/lo planes in global memory by helper
+// kernels.
 // Every mbarrier wait is bounded: on expiry the kernel records CQR_ETIMEOUT, stops issuing,
 // waits (bounded) for its own copies, frees TMEM and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -50,41 +63,51 @@ constexpr int BN = 128;       // UMMA N (TMEM columns)
 template <int U>
 constexpr int tmem_cols() { return 2 * U * BN; }
 constexpr int kEpiWarps = 8;  // two per TMEM lane quarter, each draining half the columns
-constexpr int kThreads = 32 * (4 + kEpiWarps);
 constexpr int kMaxSplits = 16;
 constexpr uint32_t kTileBytesA = BM * 128;  // 16 KB: 128 rows of one 128-byte swizzle row
 constexpr uint32_t kTileBytesB = BN * 128;  // 16 KB
 
-// Operand type of the MMAs: TF32 (kind::tf32) or BF16 (kind::f16 with BF16 inputs).  One stage
-// of K is one 128-byte swizzle row of the operand type, 32 TF32 or 64 BF16 elements; each
-// tcgen05.mma consumes 32 bytes of it (8 TF32 or 16 BF16 elements).
-template <bool BF>
+// Operand type of the MMAs: TF32 (kind::tf32), BF16 or FP16 (kind::f16, A and B of the same
+// type).  One stage of K is one 128-byte swizzle row of the operand type, 32 TF32 or 64 16-bit
+// elements; each tcgen05.mma consumes 32 bytes of it (8 TF32 or 16 16-bit elements).
+enum Kind { kTF32 = 0, kBF16 = 1, kF16 = 2 };
+template <int KD>
 struct Op {
-  static constexpr int KE = BF ? 64 : 32;
-  static constexpr int UK = BF ? 16 : 8;
+  static constexpr int KE = KD == kTF32 ? 32 : 64;
+  static constexpr int UK = KD == kTF32 ? 8 : 16;
 };
 
-// Instruction descriptor: D FP32, both operands K-major, N and M encoded; A/B format TF32
-// (kind::tf32) or BF16 (kind::f16, A and B of the same type).
-template <bool BF>
+// Warps 2 and 3 split the raw B tile.  FP16 adds two more after the epilogue's (one row of the
+// tile per thread), since a stage's products take half as long per element as in TF32; launches
+// without a split keep the registers for the epilogue instead.
+template <int KD, bool SB>
+struct Warps {
+  static constexpr int kSplit = KD == kF16 && SB ? 4 : 2;
+  static constexpr int kThreads = 32 * (2 + kSplit + kEpiWarps);
+};
+
+// Instruction descriptor: D FP32, both operands K-major, N and M encoded; A/B format FP16 (0),
+// BF16 (1) or TF32 (2).
+template <int KD>
 constexpr uint32_t idesc() {
-  return (1u << 4) | ((BF ? 1u : 2u) << 7) | ((BF ? 1u : 2u) << 10) |
-         ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+  constexpr uint32_t fmt = KD == kTF32 ? 2u : KD == kBF16 ? 1u : 0u;
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) |
+         ((uint32_t)(BM >> 4) << 24);
 }
 
-template <bool BF>
+template <int KD>
 __device__ __forceinline__ void mma_op(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accum) {
-  if (BF)
+  if (KD != kTF32)
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc<true>()), "r"(accum)
+        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc<KD>()), "r"(accum)
         : "memory");
   else
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc<false>()), "r"(accum)
+        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc<KD>()), "r"(accum)
         : "memory");
 }
 
@@ -103,7 +126,6 @@ struct TcMaps {
 
 struct TcJob {
   int nprod;          // 1 (TF32) or 3 (3xTF32)
-  int split_b_smem;   // 1: B arrives raw and is split in shared memory
   int epi;            // 0: store partial P[s] ; 1: C -= D
   int prefetch_c;     // epi 1: prefetch each output tile into L2 when its loads start
   int pair_n;         // B from planes: work units of two N tiles when n_tiles is even
@@ -119,6 +141,11 @@ struct TcJob {
   float* out;         // epi 0: P base; epi 1: C base (already offset to column j0)
   int64_t ldo;        // leading dimension of out
   int64_t split_stride;  // epi 0: elements between split partials
+  // FP16 operands: raw B rows are multiplied by bscale (nullptr: bconst) before the split, the
+  // epilogue of C -= D multiplies D by oconst and, column by column, by oinv (nullptr: 1)
+  const float* bscale;
+  const float* oinv;
+  float bconst, oconst;
   int* status;
 };
 
@@ -144,15 +171,17 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // even): the B tile is loaded (and split) once for both, and two accumulators are formed.
 // NP = 2: a pair of adjacent N tiles on the same M tile (n_tiles even, B from planes): the A
 // tiles are loaded once for both.  MP NP <= 2.
-template <bool BF, int STAGES, int NA, int NB, int MP, int NP>
-__global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__ TcMaps maps,
+// SB: B arrives as raw FP32 and is split in shared memory.
+template <int KD, bool SB, int STAGES, int NA, int NB, int MP, int NP>
+__global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __grid_constant__ TcMaps maps,
                                                           const TcJob job) {
-  static_assert(MP * NP <= 2, "at most two accumulators per buffer");
+  static_assert(MP * NP <= 2 && (!SB || NP == 1), "at most two accumulators per buffer");
   using S = Smem<STAGES, NA, NB, MP, NP>;
   constexpr int kAcc = MP * NP;  // accumulators per work unit
   constexpr int kTmemCols = tmem_cols<kAcc>();
-  constexpr int BK = Op<BF>::KE;
-  constexpr int UMMA_K = Op<BF>::UK;
+  constexpr bool BF = KD != kTF32;  // 16-bit operands
+  constexpr int BK = Op<KD>::KE;
+  constexpr int UMMA_K = Op<KD>::UK;
   extern __shared__ __align__(1024) unsigned char smraw[];
   const uint32_t base_u = su32(smraw);
   const uint32_t tiles_u = (base_u + 1023u) & ~1023u;
@@ -170,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
   // allocation)
   CQR_CHECK(job.ldo >= job.mrows && (int64_t)job.m_tiles * BM >= job.mrows &&
                 (int64_t)job.n_tiles * BN >= job.ncols && job.m_tiles % MP == 0 &&
-                job.n_tiles % NP == 0 && (NP == 1 || !job.split_b_smem), 401);
+                job.n_tiles % NP == 0 && (NP == 1 || !SB), 401);
   const int mu = job.m_tiles / MP;  // work units along M
   const int total_tiles = mu * (job.n_tiles / NP) * job.splits;
   const int nkb_full = (int)(job.kchunk / BK);
@@ -178,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&ready[s], 64);
+      mbar_init(&ready[s], 32 * Warps<KD, SB>::kSplit);
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -239,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
           const int yb = (int)(job.b_row0 + (int64_t)nt * BN);
           // raw FP32 B for the in-smem split: one 32-element box (TF32) or two (BF16: 64
           // elements of K, split in place into the BF16 hi and lo tiles)
-          const int nb_load = job.split_b_smem ? (BF ? 2 : 1) : NB;
+          const int nb_load = SB ? (BF ? 2 : 1) : NB;
           mbar_expect_tx(&full[s], MP * NA * kTileBytesA + NP * nb_load * kTileBytesB);
 #pragma unroll
           for (int m = 0; m < MP; ++m)
@@ -248,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
 #pragma unroll
           for (int n = 0; n < NP; ++n)
             for (int p = 0; p < nb_load; ++p) {
-              const bool raw = job.split_b_smem;
+              const bool raw = SB;
               tma_load_2d(st + MP * NA * kTileBytesA + (n * NB + p) * kTileBytesB,
                           raw ? &maps.b[0] : &maps.b[p], raw ? x + 32 * p : x, yb + n * BN,
                           &full[s]);
@@ -277,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
         bool ok = true;
         for (int kb = 0; kb < nk; ++kb, ++it) {
           const int s = it % STAGES;
-          uint64_t* gate = job.split_b_smem ? &ready[s] : &full[s];
+          uint64_t* gate = SB ? &ready[s] : &full[s];
           if (!mbar_wait(gate, (it / STAGES) & 1, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint32_t st = tiles_u + s * S::kStageBytes;
@@ -293,10 +322,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
                 const uint32_t a_hi = st + m * NA * kTileBytesA, a_lo = a_hi + kTileBytesA;
                 const uint32_t b_hi = st + MP * NA * kTileBytesA + n * NB * kTileBytesB;
                 const uint32_t b_lo = b_hi + kTileBytesB;
-                mma_op<BF>(am, sdesc(a_hi + off), sdesc(b_hi + off), acc0);
+                mma_op<KD>(am, sdesc(a_hi + off), sdesc(b_hi + off), acc0);
                 if (job.nprod == 3) {
-                  mma_op<BF>(am, sdesc(a_hi + off), sdesc(b_lo + off), 1u);
-                  mma_op<BF>(am, sdesc(a_lo + off), sdesc(b_hi + off), 1u);
+                  mma_op<KD>(am, sdesc(a_hi + off), sdesc(b_lo + off), 1u);
+                  mma_op<KD>(am, sdesc(a_lo + off), sdesc(b_hi + off), 1u);
                 }
               }
           }
@@ -306,13 +335,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
         mma_commit(&acc_full[buf]);
       }
     }
-  } else if (warp == 2 || warp == 3) {
-    if (job.split_b_smem) {
-      const int tt = threadIdx.x - 64;  // 0..63
+  } else if (warp < 4 || warp >= 4 + kEpiWarps) {
+    if constexpr (SB) {
+      const int tt = threadIdx.x - (warp < 4 ? 64 : 32 * (2 + kEpiWarps));
       int it = 0;
       for (int t = blockIdx.x; t < total_tiles && !*abort_flag; t += gridDim.x) {
         const int split = t % job.splits;
         const int nk = kblocks(split);
+        float sc = job.bconst;  // FP16: the scale of this thread's row of the B tile
+        if (KD == kF16 && job.bscale) {
+          const int64_t j = (int64_t)(t / job.splits / mu) * NP * BN + tt;
+          sc = j < job.ncols ? job.bscale[j] : 1.f;
+        }
         bool ok = true;
         for (int kb = 0; kb < nk; ++kb, ++it) {
           const int s = it % STAGES;
@@ -334,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
             // row r of the two raw FP32 tiles (K 0..31 and 32..63, 16-byte chunks swizzled by
             // r % 8) becomes row r of the BF16 hi tile (first 16 KB) and lo tile (second):
             // a thread reads both raw rows before writing, and no other thread touches row r
-            for (int r = tt; r < BN; r += 64) {
+            for (int r = tt; r < BN; r += 32 * Warps<KD, SB>::kSplit) {
               float v[64];
 #pragma unroll
               for (int c = 0; c < 16; ++c) {
@@ -348,6 +382,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                   const float a0 = v[8 * c + 2 * q], a1 = v[8 * c + 2 * q + 1];
+                  if constexpr (KD == kF16) {
+                    const float x0 = a0 * sc, x1 = a1 * sc;
+                    const __half2 h = __floats2half2_rn(x0, x1);
+                    const float2 f = __half22float2(h);
+                    const __half2 l = __floats2half2_rn(x0 - f.x, x1 - f.y);
+                    memcpy(&hw[q], &h, 4);
+                    memcpy(&lw[q], &l, 4);
+                    continue;
+                  }
                   const __nv_bfloat16 h0 = __float2bfloat16_rn(a0), h1 = __float2bfloat16_rn(a1);
                   const __nv_bfloat16 l0 = __float2bfloat16_rn(a0 - __bfloat162float(h0));
                   const __nv_bfloat16 l1 = __float2bfloat16_rn(a1 - __bfloat162float(h1));
@@ -395,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = 0.f;
         const int64_t col0 = (int64_t)(nt + n) * BN + c * 32;
-        if (job.epi == 0) {
+        if (job.epi == 0 || (KD == kF16 && SB)) {
           float* o = job.out + (int64_t)split * job.split_stride;
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
@@ -403,6 +446,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
             if (row_ok && col < job.ncols) o[row + col * job.ldo] = v[i];
           }
         } else {
+          // the columns' factors, one per lane, before the loads of the output tile
+          float inv = 1.f;
+          if (KD == kF16 && job.oinv && col0 + lane < job.ncols) inv = job.oinv[col0 + lane];
           float old[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
@@ -412,6 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const int64_t col = col0 + i;
+            if (KD == kF16) v[i] = v[i] * job.oconst * __shfl_sync(~0u, inv, i);
             if (row_ok && col < job.ncols) job.out[row + col * job.ldo] = old[i] - v[i];
           }
         }
@@ -440,10 +487,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
 // finished panel is also copied into the row-major planes of all computed columns
 // (Qr[r * ldrow + kb + k]), the K-major operand of the block reorthogonalisation.
 // Operand planes: x = hi + lo with hi = rna_tf32(x) (TF32; hi = x with one product, the MMA
-// reads TF32 from the FP32 word) or hi = bf16_rn(x), lo = bf16_rn(x - hi) (BF16).
+// reads TF32 from the FP32 word) or hi = rn(x), lo = rn(x - hi) in BF16 or FP16 (there x is
+// scaled: by cscale[k] where given, else by scale).
 __device__ __forceinline__ void hilo(float x, int nplanes, float& h, float& l) {
   h = nplanes == 2 ? tf32_hi(x) : x;
   l = x - h;
+}
+__device__ __forceinline__ void hilo(float x, int, __half& h, __half& l) {
+  h = __float2half_rn(x);
+  l = __float2half_rn(x - __half2float(h));
 }
 __device__ __forceinline__ void hilo(float x, int, __nv_bfloat16& h, __nv_bfloat16& l) {
   h = __float2bfloat16_rn(x);
@@ -460,7 +512,8 @@ __global__ void __launch_bounds__(256) k_split_panel(const float* __restrict__ Q
                                                      P* __restrict__ Ak_lo, int64_t ldk,
                                                      P* __restrict__ At_hi, P* __restrict__ At_lo,
                                                      P* __restrict__ Qr_hi, P* __restrict__ Qr_lo,
-                                                     int64_t ldrow, int64_t kb) {
+                                                     int64_t ldrow, int64_t kb, float scale,
+                                                     const float* __restrict__ cscale) {
   __shared__ P sh[32][33], sl[32][33];
   pdl_wait();
   pdl_trigger();
@@ -473,7 +526,7 @@ __global__ void __launch_bounds__(256) k_split_panel(const float* __restrict__ Q
     const int k = k0 + ty + 8 * i;
     const float x = (r < M && k < bk) ? Q[r + (int64_t)k * ldq] : 0.f;
     P h, l;
-    hilo(x, nplanes, h, l);
+    hilo(x * (cscale && k < bk ? cscale[k] : scale), nplanes, h, l);
     if (r < M && k < ak_cols) {
       if (Ak_hi) Ak_hi[r + (int64_t)k * ldk] = h;
       if (Ak_lo && nplanes == 2) Ak_lo[r + (int64_t)k * ldk] = l;
@@ -502,7 +555,8 @@ __global__ void __launch_bounds__(256) k_split_panel(const float* __restrict__ Q
 // C -= sum_s P[s] in a fixed order of s (split-K partials of a C -= A B update; P[s] is
 // mrows x ncols column-major with leading dimension mrows).
 __global__ void k_tc_sub_partials(const float* __restrict__ P, int splits, int64_t mrows,
-                                  int64_t ncols, float* __restrict__ C, int64_t ldc) {
+                                  int64_t ncols, float* __restrict__ C, int64_t ldc, float oconst,
+                                  const float* __restrict__ oinv) {
   pdl_wait();
   pdl_trigger();
   const int64_t total = mrows * ncols;
@@ -512,7 +566,55 @@ __global__ void k_tc_sub_partials(const float* __restrict__ P, int splits, int64
     const int64_t r = idx % mrows, c = idx / mrows;
     float s = 0.f;
     for (int sp = 0; sp < splits; ++sp) s += __ldcs(P + sp * stride + idx);
-    C[r + c * ldc] -= s;
+    C[r + c * ldc] -= oinv ? s * oconst * oinv[c] : s * oconst;
+  }
+}
+
+// FP16 scales of `ncols` columns of C (M rows): cs[j] = the power of two that takes the 2-norm
+// of column j into [2^9, 2^10), ci[j] = 1 / cs[j]; 1 for a column that is zero or not finite.
+// One CTA per column; the largest magnitude first, so that the sum of squares cannot overflow
+// or vanish (the second reading comes from the caches).
+__global__ void __launch_bounds__(256) k_col_scale(const float* __restrict__ C, int64_t ldc, int64_t M,
+                                                   float* __restrict__ cs, float* __restrict__ ci) {
+  __shared__ float red[8];
+  pdl_wait();
+  pdl_trigger();
+  const float* c = C + (int64_t)blockIdx.x * ldc;
+  const int tid = threadIdx.x;
+  float m = 0.f;
+  for (int64_t r = tid; r < M; r += 256) m = fmaxf(m, fabsf(c[r]));
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(~0u, m, o));
+  if ((tid & 31) == 0) red[tid >> 5] = m;
+  __syncthreads();
+  m = red[0];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w]);
+  __syncthreads();
+  int e = 0;
+  const bool plain = m > 0.f && m <= 3.402823466e38f;
+  if (plain) frexpf(m, &e);  // m in [2^(e-1), 2^e)
+  // x 2^-e in two exact steps, so that neither factor leaves the range
+  const float s1 = ldexpf(1.f, -(e / 2)), s2 = ldexpf(1.f, -(e - e / 2));
+  float q = 0.f;
+  for (int64_t r = tid; r < M; r += 256) {
+    const float x = c[r] * s1 * s2;
+    q += x * x;
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(~0u, q, o);
+  if ((tid & 31) == 0) red[tid >> 5] = q;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < 8; ++w) q += red[w];
+    float s = 1.f;
+    if (plain && q <= 3.402823466e38f) {
+      int eq;
+      frexpf(sqrtf(q), &eq);  // the norm lies in [2^(e+eq-1), 2^(e+eq))
+      s = ldexpf(1.f, min(126, max(-120, 10 - (e + eq))));
+    }
+    cs[blockIdx.x] = s;
+    ci[blockIdx.x] = 1.f / s;
   }
 }
 
@@ -522,7 +624,8 @@ template <typename P>
 __global__ void __launch_bounds__(256) k_refresh_rect(const float* __restrict__ Q, int64_t ldq,
                                                       int64_t r0, int nr, int64_t c0, int nc,
                                                       int nplanes, P* __restrict__ Qr_hi,
-                                                      P* __restrict__ Qr_lo, int64_t ldrow) {
+                                                      P* __restrict__ Qr_lo, int64_t ldrow,
+                                                      float scale) {
   __shared__ P sh[32][33], sl[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int rb = blockIdx.x * 32, cb = blockIdx.y * 32;
@@ -530,7 +633,7 @@ __global__ void __launch_bounds__(256) k_refresh_rect(const float* __restrict__ 
   for (int u = 0; u < 4; ++u) {
     const int r = rb + tx, c = cb + ty + 8 * u;
     P h, l;
-    hilo((r < nr && c < nc) ? Q[r0 + r + (c0 + c) * ldq] : 0.f, nplanes, h, l);
+    hilo((r < nr && c < nc) ? Q[r0 + r + (c0 + c) * ldq] * scale : 0.f, nplanes, h, l);
     sh[ty + 8 * u][tx] = h;
     sl[ty + 8 * u][tx] = l;
   }
@@ -554,7 +657,8 @@ __global__ void __launch_bounds__(256) k_tc_reduce_t(const float* __restrict__ P
                                                      int64_t split_stride, int64_t ldp, int bk,
                                                      int64_t kb, int64_t kbp, float* __restrict__ R,
                                                      int64_t ldr, int nplanes, PT* __restrict__ Sh,
-                                                     PT* __restrict__ Sl, int64_t ldrow) {
+                                                     PT* __restrict__ Sl, int64_t ldrow, float oconst,
+                                                     const float* __restrict__ oinv) {
   __shared__ float tile[32][33];
   pdl_wait();
   pdl_trigger();
@@ -568,7 +672,7 @@ __global__ void __launch_bounds__(256) k_tc_reduce_t(const float* __restrict__ P
     float s = 0.f;
     if (i < bk && j < kb)
       for (int sp = 0; sp < splits; ++sp) s += P[sp * split_stride + i + j * ldp];
-    tile[ty + 8 * u][tx] = s;
+    tile[ty + 8 * u][tx] = s * oconst;
   }
   __syncthreads();
 #pragma unroll
@@ -577,7 +681,7 @@ __global__ void __launch_bounds__(256) k_tc_reduce_t(const float* __restrict__ P
     const int64_t j = j0 + tx;
     if (i >= bk || j >= kbp) continue;
     const float s = tile[tx][ty + 8 * u];
-    if (j < kb) R[j + (kb + i) * ldr] += s;
+    if (j < kb) R[j + (kb + i) * ldr] += oinv ? s * oinv[i] : s;
     PT h, l;
     hilo(s, nplanes, h, l);
     Sh[j + i * ldrow] = h;
@@ -590,7 +694,8 @@ __global__ void __launch_bounds__(256) k_tc_reduce_t(const float* __restrict__ P
 template <typename PT>
 __global__ void k_tc_reduce(const float* __restrict__ P, int splits, int64_t split_stride, int64_t ldp,
                             int bk, int bkp, int64_t w, float* __restrict__ R, int64_t ldr,
-                            int nplanes, PT* __restrict__ Bh, PT* __restrict__ Bl) {
+                            int nplanes, PT* __restrict__ Bh, PT* __restrict__ Bl, float oconst,
+                            const float* __restrict__ oinv) {
   pdl_wait();
   pdl_trigger();
   const int64_t total = (int64_t)bkp * w;
@@ -600,7 +705,8 @@ __global__ void k_tc_reduce(const float* __restrict__ P, int splits, int64_t spl
     float s = 0.f;
     if (i < bk) {
       for (int sp = 0; sp < splits; ++sp) s += P[sp * split_stride + i + j * ldp];
-      R[i + j * ldr] = s;
+      s *= oconst;
+      R[i + j * ldr] = oinv ? s * oinv[j] : s;
     }
     PT h, l;
     hilo(s, nplanes, h, l);
@@ -615,8 +721,8 @@ __global__ void k_tc_reduce(const float* __restrict__ P, int splits, int64_t spl
 struct TcGemm {
   int mode;           // CQR_MMA_TF32 | _3XTF32 | _BF16 | _BF16X3
   int nplanes;        // 1 or 2
-  bool bf;            // operand planes in BF16 (kind::f16) rather than TF32-in-FP32
-  int KE;             // K elements per stage (32 TF32, 64 BF16)
+  int kind;           // operand type of the planes and the MMAs (Kind)
+  int KE;             // K elements per stage (32 TF32, 64 16-bit)
   size_t pe;          // bytes per plane element
   int64_t M, N, b, bkp, ldq, ldk;
   float* Q;
@@ -625,6 +731,7 @@ struct TcGemm {
   void *Ak_hi[2], *Ak_lo[2], *At_hi[2], *At_lo[2], *Bh[2], *Bl[2];
   float* P[2];
   void *Qr_hi, *Qr_lo, *Sh, *Sl;   // block reorthogonalisation operands
+  float *cs, *ci;                  // FP16: scales of the N columns and their inverses
   int64_t n, ldrow;
   int num_sms;
   int* status;
@@ -655,7 +762,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder() {
   return fn;
 }
 
-bool encode_2d(CUtensorMap* tm, void* base, bool bf, uint64_t inner, uint64_t outer,
+bool encode_2d(CUtensorMap* tm, void* base, int kind, uint64_t inner, uint64_t outer,
                uint64_t row_bytes, uint32_t box_inner, uint32_t box_outer) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = encoder();
   if (!enc) return false;
@@ -663,8 +770,10 @@ bool encode_2d(CUtensorMap* tm, void* base, bool bf, uint64_t inner, uint64_t ou
   cuuint64_t strides[1] = {row_bytes};
   cuuint32_t box[2] = {box_inner, box_outer};
   cuuint32_t es[2] = {1, 1};
-  CUresult r = enc(tm, bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                   base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  CUresult r = enc(tm, kind == kTF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                : kind == kBF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+                   2, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
@@ -689,15 +798,16 @@ cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <bool BF, int STAGES, int NA, int NB, int MP = 1, int NP = 1>
+template <int KD, bool SB, int STAGES, int NA, int NB, int MP = 1, int NP = 1>
 cudaError_t launch_gemm(const TcMaps& maps, const TcJob& job, int max_ctas, cudaStream_t st, bool pdl) {
   using S = Smem<STAGES, NA, NB, MP, NP>;
-  const void* fn = (const void*)k_tc_gemm<BF, STAGES, NA, NB, MP, NP>;
+  const void* fn = (const void*)k_tc_gemm<KD, SB, STAGES, NA, NB, MP, NP>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kTotal);
   if (e != cudaSuccess) return e;
   const int tiles = job.m_tiles / MP * (job.n_tiles / NP) * job.splits;
   const int grid = std::max(1, std::min(tiles, max_ctas));
-  return launch_k(k_tc_gemm<BF, STAGES, NA, NB, MP, NP>, dim3(grid), dim3(kThreads), S::kTotal, st,
+  return launch_k(k_tc_gemm<KD, SB, STAGES, NA, NB, MP, NP>, dim3(grid), dim3(Warps<KD, SB>::kThreads),
+                  S::kTotal, st,
                   pdl, maps, job);
 }
 
@@ -705,12 +815,12 @@ cudaError_t launch_gemm(const TcMaps& maps, const TcJob& job, int max_ctas, cuda
 // the panel spans an even number of them (b = 256): the B tile is then loaded and split once
 // for both halves of the panel, which halves the B traffic into shared memory per flop.
 // CQR_GEMM_PAIR=0 keeps one M tile per work unit.
-bool pair_m_tiles(bool three, bool bf, bool split, int m_tiles) {
+bool pair_m_tiles(const TcGemm* t, bool split, int m_tiles) {
   static const int env = [] {
     const char* e = getenv("CQR_GEMM_PAIR");
     return e ? atoi(e) : 1;
   }();
-  return env != 0 && three && !bf && split && m_tiles % 2 == 0;
+  return env != 0 && t->kind == kF16 && split && m_tiles % 2 == 0;
 }
 
 // Launches whose B comes from planes (GEMM2 and the block pass's second product) take pairs of
@@ -724,8 +834,8 @@ int npair_level() {
   }();
   return env;
 }
-bool pair_n_tiles(bool three, bool bf, bool split, const TcJob& job) {
-  return job.pair_n && three && !bf && !split && job.n_tiles % 2 == 0;
+bool pair_n_tiles(const TcGemm* t, bool split, const TcJob& job) {
+  return job.pair_n && t->kind == kF16 && !split && job.n_tiles % 2 == 0;
 }
 
 // One launch of the tensor-core kernel in the variant of the handle's mode.  split: B arrives
@@ -735,26 +845,44 @@ bool pair_n_tiles(bool three, bool bf, bool split, const TcJob& job) {
 // FP32 B of 64 K elements).
 cudaError_t launch_mode(const TcGemm* t, bool split, const TcMaps& maps, const TcJob& job,
                         cudaStream_t st, int max_ctas = 0) {
-  const bool three = t->nplanes == 2;
   const int mc = max_ctas > 0 ? std::min(max_ctas, t->num_sms) : t->num_sms;
   const bool pdl = t->pdl && st == t->pdl_st;
-  if (!t->bf) {
-    if (pair_m_tiles(three, false, split, job.m_tiles))
-      return launch_gemm<false, 2, 2, 2, 2>(maps, job, mc, st, pdl);
-    if (pair_n_tiles(three, false, split, job))
-      return launch_gemm<false, 2, 2, 2, 1, 2>(maps, job, mc, st, pdl);
-    return three ? launch_gemm<false, 3, 2, 2>(maps, job, mc, st, pdl)
-                 : launch_gemm<false, 6, 1, 1>(maps, job, mc, st, pdl);
+  if (t->kind == kF16) {
+    if (pair_m_tiles(t, split, job.m_tiles)) return launch_gemm<kF16, true, 2, 2, 2, 2>(maps, job, mc, st, pdl);
+    if (pair_n_tiles(t, split, job)) return launch_gemm<kF16, false, 2, 2, 2, 1, 2>(maps, job, mc, st, pdl);
+    return split ? launch_gemm<kF16, true, 3, 2, 2>(maps, job, mc, st, pdl)
+                 : launch_gemm<kF16, false, 3, 2, 2>(maps, job, mc, st, pdl);
   }
-  if (three) return launch_gemm<true, 3, 2, 2>(maps, job, mc, st, pdl);
-  return split ? launch_gemm<true, 4, 1, 2>(maps, job, mc, st, pdl)
-               : launch_gemm<true, 6, 1, 1>(maps, job, mc, st, pdl);
+  if (t->kind == kTF32) return launch_gemm<kTF32, false, 6, 1, 1>(maps, job, mc, st, pdl);
+  if (t->nplanes == 2)
+    return split ? launch_gemm<kBF16, true, 3, 2, 2>(maps, job, mc, st, pdl)
+                 : launch_gemm<kBF16, false, 3, 2, 2>(maps, job, mc, st, pdl);
+  return split ? launch_gemm<kBF16, true, 4, 1, 2>(maps, job, mc, st, pdl)
+               : launch_gemm<kBF16, false, 6, 1, 1>(maps, job, mc, st, pdl);
 }
 
 template <typename P>
 P* pl(void* p) { return static_cast<P*>(p); }
 
 int64_t round_to(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
+
+int kind_of(int mode) {
+  return mode == CQR_MMA_3XTF32 ? kF16 : mode == CQR_MMA_TF32 ? kTF32 : kBF16;
+}
+
+// FP16 scale of the orthonormal columns: |q| <= 1, with room for a factor of 16.
+constexpr float kQScale = 4096.f;
+float q_scale(const TcGemm* t) { return t->kind == kF16 ? kQScale : 1.f; }
+float q_inv(const TcGemm* t) { return t->kind == kF16 ? 1.f / kQScale : 1.f; }
+const float* inv_of(const TcGemm* t, int64_t j) { return t->kind == kF16 ? t->ci + j : nullptr; }
+
+// f(value of the plane type)
+template <typename F>
+cudaError_t with_plane(const TcGemm* t, F f) {
+  if (t->kind == kF16) return f(__half{});
+  if (t->kind == kBF16) return f(__nv_bfloat16{});
+  return f(float{});
+}
 
 }  // namespace
 
@@ -764,9 +892,9 @@ bool tc_available() { return true; }
 size_t tc_panel_bytes(int64_t, int) { return 0; }
 
 size_t tc_workspace_bytes(int mode, int64_t M, int64_t N, int64_t n, int b, int reorth_block) {
-  const bool bf = mode == CQR_MMA_BF16 || mode == CQR_MMA_BF16X3;
-  const size_t pe = bf ? 2 : 4;
-  const int64_t KE = bf ? 64 : 32;
+  const bool w16 = kind_of(mode) != kTF32;
+  const size_t pe = w16 ? 2 : 4;
+  const int64_t KE = w16 ? 64 : 32;
   const int64_t bkp = round_to(b, KE);
   const int64_t ldk = round_to(M, 32);
   const int64_t akc = std::max<int64_t>(bkp, round_to(b, BM));
@@ -780,6 +908,7 @@ size_t tc_workspace_bytes(int mode, int64_t M, int64_t N, int64_t n, int b, int 
     s += 2 * al256((size_t)M * ldrow * pe);      // row-major computed columns hi/lo
     s += 2 * al256((size_t)ldrow * akc * pe);    // S planes
   }
+  if (kind_of(mode) == kF16) s += 2 * al256((size_t)N * 4);  // column scales
   return s;
 }
 
@@ -788,10 +917,10 @@ TcGemm* tc_create(int mode, int64_t M, int64_t N, int64_t n, int64_t b, float* Q
   TcGemm* t = new (std::nothrow) TcGemm();
   if (!t) return nullptr;
   t->mode = mode;
-  t->bf = mode == CQR_MMA_BF16 || mode == CQR_MMA_BF16X3;
+  t->kind = kind_of(mode);
   t->nplanes = (mode == CQR_MMA_3XTF32 || mode == CQR_MMA_BF16X3) ? 2 : 1;
-  t->KE = t->bf ? 64 : 32;
-  t->pe = t->bf ? 2 : 4;
+  t->KE = t->kind == kTF32 ? 32 : 64;
+  t->pe = t->kind == kTF32 ? 4 : 2;
   t->M = M;
   t->N = N;
   t->b = b;
@@ -829,23 +958,28 @@ TcGemm* tc_create(int mode, int64_t M, int64_t N, int64_t n, int64_t b, float* Q
       return nullptr;
     }
   }
-  const bool bf = t->bf;
+  t->cs = t->ci = nullptr;
+  if (t->kind == kF16) {
+    t->cs = static_cast<float*>(take((size_t)N * 4));
+    t->ci = static_cast<float*>(take((size_t)N * 4));
+  }
+  const int kd = t->kind;
   const uint32_t KE = (uint32_t)t->KE;
   bool ok = true;
-  ok &= encode_2d(&t->tm_q_b, Q, false, (uint64_t)M, (uint64_t)N, (uint64_t)ldq * 4, 32, BN);
+  ok &= encode_2d(&t->tm_q_b, Q, kTF32, (uint64_t)M, (uint64_t)N, (uint64_t)ldq * 4, 32, BN);
   for (int u = 0; u < 2; ++u) {
-    ok &= encode_2d(&t->tm_ak[u][0], t->Ak_hi[u], bf, (uint64_t)M, (uint64_t)akc, (uint64_t)t->ldk * pe, KE, BM);
-    ok &= encode_2d(&t->tm_ak[u][1], t->Ak_lo[u], bf, (uint64_t)M, (uint64_t)akc, (uint64_t)t->ldk * pe, KE, BM);
-    ok &= encode_2d(&t->tm_at[u][0], t->At_hi[u], bf, (uint64_t)t->bkp, (uint64_t)M, (uint64_t)t->bkp * pe, KE, BM);
-    ok &= encode_2d(&t->tm_at[u][1], t->At_lo[u], bf, (uint64_t)t->bkp, (uint64_t)M, (uint64_t)t->bkp * pe, KE, BM);
-    ok &= encode_2d(&t->tm_bh[u][0], t->Bh[u], bf, (uint64_t)t->bkp, (uint64_t)N, (uint64_t)t->bkp * pe, KE, BN);
-    ok &= encode_2d(&t->tm_bh[u][1], t->Bl[u], bf, (uint64_t)t->bkp, (uint64_t)N, (uint64_t)t->bkp * pe, KE, BN);
+    ok &= encode_2d(&t->tm_ak[u][0], t->Ak_hi[u], kd, (uint64_t)M, (uint64_t)akc, (uint64_t)t->ldk * pe, KE, BM);
+    ok &= encode_2d(&t->tm_ak[u][1], t->Ak_lo[u], kd, (uint64_t)M, (uint64_t)akc, (uint64_t)t->ldk * pe, KE, BM);
+    ok &= encode_2d(&t->tm_at[u][0], t->At_hi[u], kd, (uint64_t)t->bkp, (uint64_t)M, (uint64_t)t->bkp * pe, KE, BM);
+    ok &= encode_2d(&t->tm_at[u][1], t->At_lo[u], kd, (uint64_t)t->bkp, (uint64_t)M, (uint64_t)t->bkp * pe, KE, BM);
+    ok &= encode_2d(&t->tm_bh[u][0], t->Bh[u], kd, (uint64_t)t->bkp, (uint64_t)N, (uint64_t)t->bkp * pe, KE, BN);
+    ok &= encode_2d(&t->tm_bh[u][1], t->Bl[u], kd, (uint64_t)t->bkp, (uint64_t)N, (uint64_t)t->bkp * pe, KE, BN);
   }
   if (reorth_block) {
-    ok &= encode_2d(&t->tm_qr[0], t->Qr_hi, bf, (uint64_t)t->ldrow, (uint64_t)M, (uint64_t)t->ldrow * pe, KE, BM);
-    ok &= encode_2d(&t->tm_qr[1], t->Qr_lo, bf, (uint64_t)t->ldrow, (uint64_t)M, (uint64_t)t->ldrow * pe, KE, BM);
-    ok &= encode_2d(&t->tm_s[0], t->Sh, bf, (uint64_t)t->ldrow, (uint64_t)akc, (uint64_t)t->ldrow * pe, KE, BN);
-    ok &= encode_2d(&t->tm_s[1], t->Sl, bf, (uint64_t)t->ldrow, (uint64_t)akc, (uint64_t)t->ldrow * pe, KE, BN);
+    ok &= encode_2d(&t->tm_qr[0], t->Qr_hi, kd, (uint64_t)t->ldrow, (uint64_t)M, (uint64_t)t->ldrow * pe, KE, BM);
+    ok &= encode_2d(&t->tm_qr[1], t->Qr_lo, kd, (uint64_t)t->ldrow, (uint64_t)M, (uint64_t)t->ldrow * pe, KE, BM);
+    ok &= encode_2d(&t->tm_s[0], t->Sh, kd, (uint64_t)t->ldrow, (uint64_t)akc, (uint64_t)t->ldrow * pe, KE, BN);
+    ok &= encode_2d(&t->tm_s[1], t->Sl, kd, (uint64_t)t->ldrow, (uint64_t)akc, (uint64_t)t->ldrow * pe, KE, BN);
   }
   if (!ok) {
     delete t;
@@ -890,33 +1024,43 @@ int tc_splits(const TcGemm* t, int m1, int n1, int64_t* kchunk, int max_ctas = 0
   const int ctas = max_ctas > 0 ? std::min(max_ctas, t->num_sms) : t->num_sms;
   const int64_t kblocks = (t->M + t->KE - 1) / t->KE;
   // work units of the GEMM1-shaped launch (pairs of M tiles where launch_mode pairs them)
-  const bool three = t->nplanes == 2;
-  const int units_m = pair_m_tiles(three, t->bf, three || t->bf, m1) ? m1 / 2 : m1;
+  const int units_m = pair_m_tiles(t, true, m1) ? m1 / 2 : m1;
   *kchunk = best_kchunk((int64_t)units_m * n1, kblocks, ctas, kMaxSplits) * t->KE;
   return (int)((t->M + *kchunk - 1) / *kchunk);
 }
 }  // namespace
 
-// 1. split the panel Q[:, kb : kb+bk] into the operand planes of both GEMMs (and, for a
-//    finished panel with block reorthogonalisation on, into the row-major computed columns)
-cudaError_t tc_split_panel(TcGemm* t, int64_t kb, int bk, bool finished, int buf, cudaStream_t st) {
+// Scales of all columns, before the first panel: the norms of the trailing columns only fall
+// (up to rounding) as panels are taken out of them, so the scales hold for the whole factor.
+cudaError_t tc_begin(TcGemm* t, cudaStream_t st) {
+  if (t->kind != kF16) return cudaSuccess;
+  return launch_k(k_col_scale, dim3((unsigned)t->N), dim3(256), 0, st, t->pdl && st == t->pdl_st,
+                  (const float*)t->Q, t->ldq, t->M, t->cs, t->ci);
+}
+
+namespace {
+cudaError_t split_panel(TcGemm* t, int64_t kb, int bk, bool finished, const float* cscale, int buf,
+                        cudaStream_t st) {
   const int bkp = (int)round_to(bk, t->KE);
   const int m1 = (bk + BM - 1) / BM;
   dim3 grd((unsigned)((t->M + 31) / 32), (unsigned)((std::max(bkp, m1 * BM) + 31) / 32));
   void* qh = finished ? t->Qr_hi : nullptr;
   const bool pdl = t->pdl && st == t->pdl_st;
   const float* q0 = t->Q + kb * t->ldq;
-  if (t->bf) {
-    using B16 = __nv_bfloat16;
-    return launch_k(k_split_panel<B16>, grd, dim3(256), 0, st, pdl, q0, t->ldq, t->M, bk, bkp,
-                    (int)(m1 * BM), t->nplanes, pl<B16>(t->Ak_hi[buf]), pl<B16>(t->Ak_lo[buf]), t->ldk,
-                    pl<B16>(t->At_hi[buf]), pl<B16>(t->At_lo[buf]), pl<B16>(qh), pl<B16>(t->Qr_lo),
-                    t->ldrow, kb);
-  }
-  return launch_k(k_split_panel<float>, grd, dim3(256), 0, st, pdl, q0, t->ldq, t->M, bk, bkp,
-                  (int)(m1 * BM), t->nplanes, pl<float>(t->Ak_hi[buf]), pl<float>(t->Ak_lo[buf]), t->ldk,
-                  pl<float>(t->At_hi[buf]), pl<float>(t->At_lo[buf]), pl<float>(qh), pl<float>(t->Qr_lo),
-                  t->ldrow, kb);
+  return with_plane(t, [&](auto tag) {
+    using P = decltype(tag);
+    return launch_k(k_split_panel<P>, grd, dim3(256), 0, st, pdl, q0, t->ldq, t->M, bk, bkp,
+                    (int)(m1 * BM), t->nplanes, pl<P>(t->Ak_hi[buf]), pl<P>(t->Ak_lo[buf]), t->ldk,
+                    pl<P>(t->At_hi[buf]), pl<P>(t->At_lo[buf]), pl<P>(qh), pl<P>(t->Qr_lo), t->ldrow, kb,
+                    q_scale(t), cscale);
+  });
+}
+}  // namespace
+
+// 1. split the finished panel Q[:, kb : kb+bk] into the operand planes of both GEMMs (and, with
+//    block reorthogonalisation on, into the row-major computed columns)
+cudaError_t tc_split_panel(TcGemm* t, int64_t kb, int bk, int buf, cudaStream_t st) {
+  return split_panel(t, kb, bk, true, nullptr, buf, st);
 }
 
 bool tc_has_block_reorth(const TcGemm* t) { return t->Qr_hi != nullptr; }
@@ -926,19 +1070,19 @@ bool tc_has_block_reorth(const TcGemm* t) { return t->Qr_hi != nullptr; }
 cudaError_t tc_refresh_rect(TcGemm* t, int64_t r0, int64_t nr, int64_t c0, int64_t nc, cudaStream_t st) {
   if (!t->Qr_hi || nr <= 0 || nc <= 0) return cudaSuccess;
   const dim3 grd((unsigned)((nr + 31) / 32), (unsigned)((nc + 31) / 32));
-  if (t->bf)
-    k_refresh_rect<__nv_bfloat16><<<grd, 256, 0, st>>>(t->Q, t->ldq, r0, (int)nr, c0, (int)nc, t->nplanes,
-                                                      pl<__nv_bfloat16>(t->Qr_hi),
-                                                      pl<__nv_bfloat16>(t->Qr_lo), t->ldrow);
-  else
-    k_refresh_rect<float><<<grd, 256, 0, st>>>(t->Q, t->ldq, r0, (int)nr, c0, (int)nc, t->nplanes,
-                                              pl<float>(t->Qr_hi), pl<float>(t->Qr_lo), t->ldrow);
-  return cudaGetLastError();
+  return with_plane(t, [&](auto tag) {
+    using P = decltype(tag);
+    k_refresh_rect<P><<<grd, 256, 0, st>>>(t->Q, t->ldq, r0, (int)nr, c0, (int)nc, t->nplanes,
+                                           pl<P>(t->Qr_hi), pl<P>(t->Qr_lo), t->ldrow, q_scale(t));
+    return cudaGetLastError();
+  });
 }
 
 // 2. GEMM1, split-K over the M rows: partials P[s] = Qbar^T Q[:, j0 : j0+w]
-cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int ctx, int max_ctas,
-                         cudaStream_t st) {
+namespace {
+// bscale: FP16 scales of the columns j0.. of Q (nullptr: orthonormal columns)
+cudaError_t gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, const float* bscale, int buf, int ctx,
+                      int max_ctas, cudaStream_t st) {
   const int three = t->nplanes == 2;
   const int bkp = (int)round_to(bk, t->KE);
   const int m1 = (bk + BM - 1) / BM;
@@ -953,8 +1097,7 @@ cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int 
   TcJob job{};
   job.nprod = three ? 3 : 1;
   // TF32 reads the raw FP32 words directly with one product; every other mode splits B
-  const bool split = three || t->bf;
-  job.split_b_smem = split ? 1 : 0;
+  const bool split = three || t->kind != kTF32;
   job.epi = 0;
   job.m_tiles = m1;
   job.n_tiles = n1;
@@ -969,8 +1112,16 @@ cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int 
   job.out = t->P[ctx];
   job.ldo = bkp;
   job.split_stride = (int64_t)bkp * w;
+  job.bscale = bscale;
+  job.bconst = q_scale(t);
   job.status = t->status;
   return launch_mode(t, split, maps, job, st, max_ctas);
+}
+}  // namespace
+
+cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int ctx, int max_ctas,
+                         cudaStream_t st) {
+  return gemm_rbar(t, bk, j0, w, t->kind == kF16 ? t->cs + j0 : nullptr, buf, ctx, max_ctas, st);
 }
 
 // 3. reduce the partials into R[kb.., j0..] and GEMM2's B planes
@@ -986,13 +1137,12 @@ cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, floa
   const bool pdl = t->pdl && st == t->pdl_st;
   const float* P = t->P[ctx];
   float* Rd = R + kb + j0 * ldr;
-  if (t->bf)
-    return launch_k(k_tc_reduce<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, pdl, P, splits,
-                    (int64_t)bkp * w, (int64_t)bkp, bk, bkp, w, Rd, ldr, t->nplanes,
-                    pl<__nv_bfloat16>(t->Bh[ctx]), pl<__nv_bfloat16>(t->Bl[ctx]));
-  return launch_k(k_tc_reduce<float>, dim3(blocks), dim3(256), 0, st, pdl, P, splits, (int64_t)bkp * w,
-                  (int64_t)bkp, bk, bkp, w, Rd, ldr, t->nplanes, pl<float>(t->Bh[ctx]),
-                  pl<float>(t->Bl[ctx]));
+  return with_plane(t, [&](auto tag) {
+    using P_ = decltype(tag);
+    return launch_k(k_tc_reduce<P_>, dim3(blocks), dim3(256), 0, st, pdl, P, splits, (int64_t)bkp * w,
+                    (int64_t)bkp, bk, bkp, w, Rd, ldr, t->nplanes, pl<P_>(t->Bh[ctx]),
+                    pl<P_>(t->Bl[ctx]), q_inv(t), inv_of(t, j0));
+  });
 }
 
 // 4. GEMM2: Q[:, j0 : j0+w] -= Qbar Rbar (M tiles over rows, N tiles over trailing columns)
@@ -1007,7 +1157,6 @@ cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, in
   maps.b[1] = t->tm_bh[ctx][1];
   TcJob job{};
   job.nprod = three ? 3 : 1;
-  job.split_b_smem = 0;
   job.epi = 1;
   job.m_tiles = (int)((t->M + BM - 1) / BM);
   job.n_tiles = (int)((w + BN - 1) / BN);
@@ -1026,21 +1175,33 @@ cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, in
   maps.c = t->tm_q_b;
   job.prefetch_c = 1;
   job.c_col0 = j0;
+  job.oconst = q_inv(t);
+  job.oinv = inv_of(t, j0);
   job.pair_n = npair_level() >= 2 ? 1 : 0;
   return launch_mode(t, false, maps, job, st, max_ctas);
 }
 
 // Block reorthogonalisation of panel kb .. kb+bk-1 against columns 0 .. kb-1 (four
-// launches: split the panel, S^T = Qbar^T Q[:, 0:kb] split-K on the tensor cores, reduce
+// launches, five with FP16 operands: the scales of the panel's columns as they are now, split
+// the panel, S^T = Qbar^T Q[:, 0:kb] split-K on the tensor cores, reduce
 // into R and S, Qbar -= Qrows S on the tensor cores).
 cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr, int buf,
                             cudaStream_t st, int* launches) {
   *launches = 0;
   if (!t->Qr_hi || kb <= 0) return cudaSuccess;
   *launches = 4;
-  cudaError_t e = tc_split_panel(t, kb, bk, false, buf, st);
+  cudaError_t e = cudaSuccess;
+  const float* ps = nullptr;
+  if (t->kind == kF16) {
+    ++*launches;
+    e = launch_k(k_col_scale, dim3((unsigned)bk), dim3(256), 0, st, t->pdl && st == t->pdl_st,
+                 (const float*)(t->Q + kb * t->ldq), t->ldq, t->M, t->cs + kb, t->ci + kb);
+    if (e != cudaSuccess) return e;
+    ps = t->cs + kb;
+  }
+  e = split_panel(t, kb, bk, false, ps, buf, st);
   if (e != cudaSuccess) return e;
-  e = tc_gemm_rbar(t, bk, 0, kb, buf, 0, 0, st);  // partials of S^T (bk x kb), context 0
+  e = gemm_rbar(t, bk, 0, kb, nullptr, buf, 0, 0, st);  // partials of S^T (bk x kb), context 0
   if (e != cudaSuccess) return e;
   const int KE = t->KE;
   const int bkp = (int)round_to(bk, KE);
@@ -1053,14 +1214,12 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
     const dim3 blocks((unsigned)((bk + 31) / 32), (unsigned)((kbp + 31) / 32));
     const bool pdl = t->pdl && st == t->pdl_st;
     const float* P0 = t->P[0];
-    if (t->bf)
-      e = launch_k(k_tc_reduce_t<__nv_bfloat16>, blocks, dim3(256), 0, st, pdl, P0, splits,
-                   (int64_t)bkp * kb, (int64_t)bkp, bk, kb, kbp, R, ldr, t->nplanes,
-                   pl<__nv_bfloat16>(t->Sh), pl<__nv_bfloat16>(t->Sl), t->ldrow);
-    else
-      e = launch_k(k_tc_reduce_t<float>, blocks, dim3(256), 0, st, pdl, P0, splits,
-                   (int64_t)bkp * kb, (int64_t)bkp, bk, kb, kbp, R, ldr, t->nplanes,
-                   pl<float>(t->Sh), pl<float>(t->Sl), t->ldrow);
+    e = with_plane(t, [&](auto tag) {
+      using P = decltype(tag);
+      return launch_k(k_tc_reduce_t<P>, blocks, dim3(256), 0, st, pdl, P0, splits, (int64_t)bkp * kb,
+                      (int64_t)bkp, bk, kb, kbp, R, ldr, t->nplanes, pl<P>(t->Sh), pl<P>(t->Sl),
+                      t->ldrow, q_inv(t), inv_of(t, kb));
+    });
     if (e != cudaSuccess) return e;
   }
   TcMaps maps;
@@ -1070,7 +1229,6 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
   maps.b[1] = t->tm_s[1];
   TcJob job{};
   job.nprod = t->nplanes == 2 ? 3 : 1;
-  job.split_b_smem = 0;
   job.epi = 1;
   job.m_tiles = (int)((t->M + BM - 1) / BM);
   job.n_tiles = (bk + BN - 1) / BN;
@@ -1080,7 +1238,9 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
   // depend on the schedule.
   const int64_t kblk = kbp / KE;
   job.pair_n = npair_level() >= 1 ? 1 : 0;
-  const bool np2 = pair_n_tiles(t->nplanes == 2, t->bf, false, job);
+  job.oconst = q_inv(t);
+  job.oinv = inv_of(t, kb);
+  const bool np2 = pair_n_tiles(t, false, job);
   const int tiles2 = job.m_tiles * (job.n_tiles / (np2 ? 2 : 1));
   const int64_t cap = std::min<int64_t>(kMaxSplits, (int64_t)kMaxSplits * t->bkp * t->N /
                                                         (t->M * (int64_t)bk));
@@ -1108,12 +1268,12 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
   }
   e = launch_mode(t, false, maps, job, st);
   if (e != cudaSuccess || splits2 == 1) return e;
-  *launches = 5;
+  ++*launches;
   const int64_t total = t->M * (int64_t)bk;
   const int blocks = (int)std::min<int64_t>((int64_t)t->num_sms * 8, (total + 255) / 256);
   const bool pdl = t->pdl && st == t->pdl_st;
   return launch_k(k_tc_sub_partials, dim3(blocks), dim3(256), 0, st, pdl, (const float*)t->P[0], splits2,
-                  t->M, (int64_t)bk, t->Q + kb * t->ldq, t->ldq);
+                  t->M, (int64_t)bk, t->Q + kb * t->ldq, t->ldq, q_inv(t), inv_of(t, kb));
 }
 
 // General C -= op(A) B in 3xTF32 on the tensor cores (the large products of the reverse mode).
@@ -1142,26 +1302,25 @@ cudaError_t tc_gemm_sub3(bool a_trans, const float* A, int64_t lda, const float*
     float* lo = hi + kp * M;
     const dim3 grd((unsigned)((K + 31) / 32), (unsigned)((M + 31) / 32));
     k_split_panel<float><<<grd, 256, 0, st>>>(A, lda, K, (int)M, 0, (int)M, 2, hi, lo, kp, nullptr,
-                                              nullptr, nullptr, nullptr, 0, 0);
-    ok &= encode_2d(&maps.a[0], hi, false, (uint64_t)K, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
-    ok &= encode_2d(&maps.a[1], lo, false, (uint64_t)K, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
+                                              nullptr, nullptr, nullptr, 0, 0, 1.f, nullptr);
+    ok &= encode_2d(&maps.a[0], hi, kTF32, (uint64_t)K, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
+    ok &= encode_2d(&maps.a[1], lo, kTF32, (uint64_t)K, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
   } else {
     // planes of A (M x K): row-major, row stride kp
     float* lo = hi + M * kp;
     const dim3 grd((unsigned)((M + 31) / 32), (unsigned)((kp + 31) / 32));
     k_split_panel<float><<<grd, 256, 0, st>>>(A, lda, M, (int)K, (int)kp, 0, 2, nullptr, nullptr, 0, hi,
-                                              lo, nullptr, nullptr, 0, 0);
-    ok &= encode_2d(&maps.a[0], hi, false, (uint64_t)kp, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
-    ok &= encode_2d(&maps.a[1], lo, false, (uint64_t)kp, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
+                                              lo, nullptr, nullptr, 0, 0, 1.f, nullptr);
+    ok &= encode_2d(&maps.a[0], hi, kTF32, (uint64_t)kp, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
+    ok &= encode_2d(&maps.a[1], lo, kTF32, (uint64_t)kp, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  ok &= encode_2d(&maps.b[0], const_cast<float*>(B), false, (uint64_t)K, (uint64_t)N, (uint64_t)ldb * 4, 32, BN);
+  ok &= encode_2d(&maps.b[0], const_cast<float*>(B), kTF32, (uint64_t)K, (uint64_t)N, (uint64_t)ldb * 4, 32, BN);
   maps.b[1] = maps.b[0];
   if (!ok) return cudaErrorInvalidValue;
   TcJob job{};
   job.nprod = 3;
-  job.split_b_smem = 1;
   job.epi = 1;
   job.m_tiles = (int)((M + BM - 1) / BM);
   job.n_tiles = (int)((N + BN - 1) / BN);
@@ -1177,7 +1336,7 @@ cudaError_t tc_gemm_sub3(bool a_trans, const float* A, int64_t lda, const float*
   job.ldo = ldc;
   job.split_stride = 0;
   job.status = status;
-  return launch_gemm<false, 3, 2, 2>(maps, job, num_sms, st, false);
+  return launch_gemm<kTF32, true, 3, 2, 2>(maps, job, num_sms, st, false);
 }
 
 cudaError_t bounds_take_tc(int* code, int* site) { return bounds_take_here(code, site); }
