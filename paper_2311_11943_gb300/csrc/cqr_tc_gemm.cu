@@ -1041,7 +1041,7 @@ cudaError_t tc_begin(TcGemm* t, cudaStream_t st) {
 namespace {
 cudaError_t split_panel(TcGemm* t, int64_t kb, int bk, bool finished, const float* cscale, int buf,
                         cudaStream_t st) {
-  const int bkp = (int)round_to(bk, t->KE);
+  const int bkp = (int)t->bkp;  // the planes' stride in the tensor maps, also for a narrower last panel
   const int m1 = (bk + BM - 1) / BM;
   dim3 grd((unsigned)((t->M + 31) / 32), (unsigned)((std::max(bkp, m1 * BM) + 31) / 32));
   void* qh = finished ? t->Qr_hi : nullptr;
@@ -1084,7 +1084,7 @@ namespace {
 cudaError_t gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, const float* bscale, int buf, int ctx,
                       int max_ctas, cudaStream_t st) {
   const int three = t->nplanes == 2;
-  const int bkp = (int)round_to(bk, t->KE);
+  const int bkp = (int)t->bkp;
   const int m1 = (bk + BM - 1) / BM;
   const int n1 = (int)((w + BN - 1) / BN);
   int64_t kchunk = 0;
@@ -1127,7 +1127,7 @@ cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int 
 // 3. reduce the partials into R[kb.., j0..] and GEMM2's B planes
 cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, float* R, int64_t ldr,
                       int ctx, int max_ctas, cudaStream_t st) {
-  const int bkp = (int)round_to(bk, t->KE);
+  const int bkp = (int)t->bkp;
   const int m1 = (bk + BM - 1) / BM;
   const int n1 = (int)((w + BN - 1) / BN);
   int64_t kchunk = 0;
@@ -1149,7 +1149,7 @@ cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, floa
 cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int ctx, int max_ctas,
                            cudaStream_t st) {
   const int three = t->nplanes == 2;
-  const int bkp = (int)round_to(bk, t->KE);
+  const int64_t kk = round_to(bk, t->KE);  // planes are zero from bk to there
   TcMaps maps;
   maps.a[0] = t->tm_at[buf][0];
   maps.a[1] = t->tm_at[buf][1];
@@ -1164,8 +1164,8 @@ cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, in
   job.a_row0 = 0;
   job.b_row0 = 0;
   job.k0 = 0;
-  job.kchunk = bkp;
-  job.K = bkp;
+  job.kchunk = kk;
+  job.K = kk;
   job.mrows = t->M;
   job.ncols = w;
   job.out = t->Q + j0 * t->ldq;
@@ -1204,7 +1204,7 @@ cudaError_t tc_block_reorth(TcGemm* t, int64_t kb, int bk, float* R, int64_t ldr
   e = gemm_rbar(t, bk, 0, kb, nullptr, buf, 0, 0, st);  // partials of S^T (bk x kb), context 0
   if (e != cudaSuccess) return e;
   const int KE = t->KE;
-  const int bkp = (int)round_to(bk, KE);
+  const int bkp = (int)t->bkp;
   const int m1 = (bk + BM - 1) / BM;
   const int n1 = (int)((kb + BN - 1) / BN);
   int64_t kchunk = 0;
