@@ -28,8 +28,9 @@
 // 2^-34 of the column's norm per entry, 2^-10 of the FP32 rounding of the column itself.  Measured
 // against 64 bits: R of 8192 x 8192 1.4e-5 -> 7.7e-6, of 16384 x 2048 6.9e-6 -> 3.7e-6 relative to
 // TF32 halves (fewer roundings in the accumulators).  8192 x 8192, p = 16, b = 256, all panels:
-// Rbar 5.0 -> 2.95 ms, block pass 8.1 -> 5.4 ms, update 4.94 -> 4.38 ms (one pass over the
-// trailing columns, 1.6 ms at the copy rate; bound by the reads of C in the epilogue).
+// Rbar 5.0 -> 2.95 ms, block pass 8.1 -> 5.4 ms, update 4.94 -> 4.38 ms, and 3.52 ms
+// with C through shared memory (CT below; one pass over the trailing columns is 1.6 ms at the copy
+// rate).
 // The small operands (panel and Rbar) are split into hi/lo planes in global memory by helper
 // kernels.
 // Every mbarrier wait is bounded: on expiry the kernel records CQR_ETIMEOUT, stops issuing,
@@ -64,6 +65,9 @@ template <int U>
 constexpr int tmem_cols() { return 2 * U * BN; }
 constexpr int kEpiWarps = 8;  // two per TMEM lane quarter, each draining half the columns
 constexpr int kMaxSplits = 16;
+// C ring of an epilogue warp (CT): chunks of 32 rows x 32 columns, 4 KB
+constexpr int kCSlots = 3;
+constexpr uint32_t kCBytes = 32 * 32 * 4;
 constexpr uint32_t kTileBytesA = BM * 128;  // 16 KB: 128 rows of one 128-byte swizzle row
 constexpr uint32_t kTileBytesB = BN * 128;  // 16 KB
 
@@ -149,15 +153,17 @@ struct TcJob {
   int* status;
 };
 
-template <int STAGES, int NA, int NB, int MP = 1, int NP = 1>
+template <int STAGES, int NA, int NB, int MP = 1, int NP = 1, bool CT = false>
 struct Smem {
   // per stage: NA A tiles for each of the MP M tiles, then NB B tiles for each of the NP N
   // tiles (each 1024-byte aligned, 16 KB)
   static constexpr uint32_t kStageBytes = MP * NA * kTileBytesA + NP * NB * kTileBytesB;
   static constexpr uint32_t kTiles = STAGES * kStageBytes;
-  static constexpr uint32_t kTotal = kTiles + 1024 /*alignment*/ + 256 /*barriers*/;
-  // full/ready/empty per stage, acc_full[2], acc_empty[2], TMEM slot, abort flag
-  static_assert(STAGES * 3 * 8 + 4 * 8 + 8 <= 256, "barrier region too small");
+  static constexpr uint32_t kRing = CT ? kEpiWarps * kCSlots * kCBytes : 0;
+  static constexpr uint32_t kTotal = kTiles + kRing + 1024 /*alignment*/ + 512 /*barriers*/;
+  // full/ready/empty per stage, acc_full[2], acc_empty[2], C ring, TMEM slot, abort flag
+  static_assert(STAGES * 3 * 8 + 4 * 8 + kEpiWarps * kCSlots * 8 + 8 <= 512, "barrier region too small");
+  static_assert(kTotal <= 227 * 1024, "shared memory");
 };
 
 // Programmatic dependent launch: a kernel launched with programmatic stream serialization may
@@ -172,11 +178,17 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // NP = 2: a pair of adjacent N tiles on the same M tile (n_tiles even, B from planes): the A
 // tiles are loaded once for both.  MP NP <= 2.
 // SB: B arrives as raw FP32 and is split in shared memory.
-template <int KD, bool SB, int STAGES, int NA, int NB, int MP, int NP>
+// CT: C -= D with C through shared memory: each epilogue warp streams its chunks of C by TMA, two
+// ahead of the one at work, and stores them by TMA.  With loads to registers a warp had one chunk
+// in flight and only between its accumulator and its stores: 4096 x 4096, b = 128, 1.34 -> 1.05 ms
+// for all panels, 8192 x 8192, b = 256, 4.38 -> 3.52 ms, although the ring leaves two operand
+// stages in place of three.
+template <int KD, bool SB, int STAGES, int NA, int NB, int MP, int NP, bool CT>
 __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __grid_constant__ TcMaps maps,
                                                           const TcJob job) {
   static_assert(MP * NP <= 2 && (!SB || NP == 1), "at most two accumulators per buffer");
-  using S = Smem<STAGES, NA, NB, MP, NP>;
+  static_assert(!CT || (MP * NP == 1 && !SB && kEpiWarps == 8), "two chunks of each tile per epilogue warp");
+  using S = Smem<STAGES, NA, NB, MP, NP, CT>;
   constexpr int kAcc = MP * NP;  // accumulators per work unit
   constexpr int kTmemCols = tmem_cols<kAcc>();
   constexpr bool BF = KD != kTF32;  // 16-bit operands
@@ -186,12 +198,13 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
   const uint32_t base_u = su32(smraw);
   const uint32_t tiles_u = (base_u + 1023u) & ~1023u;
   unsigned char* tiles = smraw + (tiles_u - base_u);
-  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + S::kTiles);
+  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + S::kTiles + S::kRing);
   uint64_t* ready = full + STAGES;     // B split done (3xTF32 in-smem split)
   uint64_t* empty = ready + STAGES;
   uint64_t* acc_full = empty + STAGES;  // [2]: one per TMEM accumulator buffer
   uint64_t* acc_empty = acc_full + 2;   // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* cfull = acc_empty + 2;      // [kEpiWarps][kCSlots] (CT)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(cfull + kEpiWarps * kCSlots);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -214,6 +227,8 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
       mbar_init(&acc_full[b], 1);
       mbar_init(&acc_empty[b], kEpiWarps);
     }
+    if (CT)
+      for (int i = 0; i < kEpiWarps * kCSlots; ++i) mbar_init(&cfull[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     prefetch_tmap(&maps.a[0]);
@@ -409,6 +424,91 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
         if (!ok) break;
       }
     }
+  } else if constexpr (CT) {
+    // chunk g of this warp: 32-column chunk half + 2 (g % 2) of the CTA's unit g / 2
+    const int ew = warp & 3, half = (warp - 4) >> 2;
+    const uint32_t ring_u = tiles_u + S::kTiles + (uint32_t)(warp - 4) * kCSlots * kCBytes;
+    unsigned char* ring = tiles + S::kTiles + (size_t)(warp - 4) * kCSlots * kCBytes;
+    uint64_t* cbar = cfull + (warp - 4) * kCSlots;
+    uint32_t phase = 0, pending = 0;  // of each slot
+    // the chunk's rows and columns; whole: it goes through the ring (all its columns belong to the
+    // job; rows past M are dropped by the tensor map)
+    auto place = [&](int g, int64_t& row0, int64_t& col0) {
+      const int t = blockIdx.x + (g >> 1) * gridDim.x;
+      if (t >= total_tiles) return false;
+      row0 = (int64_t)(t % mu) * BM + ew * 32;
+      col0 = (int64_t)(t / mu) * BN + (half + 2 * (g & 1)) * 32;
+      return row0 < job.mrows && col0 + 32 <= job.ncols;
+    };
+    auto cload = [&](int g) {
+      int64_t row0, col0;
+      if (!place(g, row0, col0)) return;
+      const int s = g % kCSlots;
+      pending |= 1u << s;
+      if (lane == 0) {
+        mbar_expect_tx(&cbar[s], kCBytes);
+        tma_load_2d(ring_u + s * kCBytes, &maps.c, (int)row0, (int)(job.c_col0 + col0), &cbar[s]);
+      }
+    };
+    cload(0);
+    cload(1);
+    int tl = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tl) {
+      const int buf = tl & 1;
+      ok = __all_sync(~0u, mbar_wait(&acc_full[buf], (tl >> 1) & 1, abort_flag) ? 1 : 0);
+      if (!ok) break;
+      tc_fence_after();
+#pragma unroll 1
+      for (int u = 0; u < 2; ++u) {
+        const int g = 2 * tl + u, s = g % kCSlots, c = half + 2 * u;
+        if (lane == 0) bulk_wait_read();  // the slot of chunk g + 2 was stored from two chunks ago
+        __syncwarp();
+        cload(g + 2);
+        int64_t row0 = 0, col0 = 0;
+        const bool whole = place(g, row0, col0);
+        const int64_t row = row0 + lane;
+        float inv = 1.f;
+        if (job.oinv && col0 + lane < job.ncols) inv = job.oinv[col0 + lane];
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(buf * BN + c * 32), v);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = v[i] * job.oconst * __shfl_sync(~0u, inv, i);
+        if (whole) {
+          ok = __all_sync(~0u, mbar_wait(&cbar[s], (phase >> s) & 1, abort_flag) ? 1 : 0);
+          if (!ok) break;
+          phase ^= 1u << s;
+          pending &= ~(1u << s);
+          // column i of the chunk is one 128-byte row of the box, its 16-byte units swizzled
+          unsigned char* sl = ring + s * kCBytes + (lane & 3) * 4;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float* x = reinterpret_cast<float*>(sl + i * 128 + (((lane >> 2) ^ (i & 7)) << 4));
+            *x -= v[i];
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_2d(&maps.c, (int)row0, (int)(job.c_col0 + col0), ring_u + s * kCBytes);
+            bulk_commit();
+          }
+        } else if (row < job.mrows) {
+          for (int i = 0; i < 32; ++i)
+            if (col0 + i < job.ncols) job.out[row + (col0 + i) * job.ldo] -= v[i];
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[buf]);
+    }
+    // nothing of this warp is in flight when the CTA exits (loads: bounded)
+    for (int s = 0; s < kCSlots; ++s)
+      if (pending >> s & 1) {
+        const long long t0 = clock64();
+        while (!mbar_test(&cbar[s], (phase >> s) & 1) && clock64() - t0 < kWaitLimitCycles) {
+        }
+      }
+    if (lane == 0) bulk_wait();
   } else {
     // epilogue warps 4 .. 4+kEpiWarps-1: TMEM lanes 32 (warp % 4) .. +32 (a warp may only
     // read its own quarter of the lanes); the two warps of a quarter take alternate 32-column
@@ -738,6 +838,7 @@ struct TcGemm {
   bool pdl = false;  // launches on pdl_st use programmatic dependent launch
   cudaStream_t pdl_st = nullptr;
   CUtensorMap tm_q_b;        // Q (FP32) as GEMM1's raw B (box 32 x BN)
+  CUtensorMap tm_q_c;        // Q in chunks of 32 rows x 32 columns (CT)
   CUtensorMap tm_ak[2][2];   // [buffer][plane] panel, column-major (box KE x BM)
   CUtensorMap tm_at[2][2];   // [buffer][plane] panel, row-major (box KE x BM)
   CUtensorMap tm_bh[2][2];   // [context][plane] Rbar planes (box KE x BN)
@@ -798,15 +899,15 @@ cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <int KD, bool SB, int STAGES, int NA, int NB, int MP = 1, int NP = 1>
+template <int KD, bool SB, int STAGES, int NA, int NB, int MP = 1, int NP = 1, bool CT = false>
 cudaError_t launch_gemm(const TcMaps& maps, const TcJob& job, int max_ctas, cudaStream_t st, bool pdl) {
-  using S = Smem<STAGES, NA, NB, MP, NP>;
-  const void* fn = (const void*)k_tc_gemm<KD, SB, STAGES, NA, NB, MP, NP>;
+  using S = Smem<STAGES, NA, NB, MP, NP, CT>;
+  const void* fn = (const void*)k_tc_gemm<KD, SB, STAGES, NA, NB, MP, NP, CT>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kTotal);
   if (e != cudaSuccess) return e;
   const int tiles = job.m_tiles / MP * (job.n_tiles / NP) * job.splits;
   const int grid = std::max(1, std::min(tiles, max_ctas));
-  return launch_k(k_tc_gemm<KD, SB, STAGES, NA, NB, MP, NP>, dim3(grid), dim3(Warps<KD, SB>::kThreads),
+  return launch_k(k_tc_gemm<KD, SB, STAGES, NA, NB, MP, NP, CT>, dim3(grid), dim3(Warps<KD, SB>::kThreads),
                   S::kTotal, st,
                   pdl, maps, job);
 }
@@ -825,8 +926,7 @@ bool pair_m_tiles(const TcGemm* t, bool split, int m_tiles) {
 
 // Launches whose B comes from planes (GEMM2 and the block pass's second product) take pairs of
 // N tiles when the job asks for it (TcJob::pair_n) and n_tiles is even: the A tiles are then
-// loaded once for both.  CQR_GEMM_NPAIR: 0 never, 1 the block pass's second product only
-// (the default), 2 also GEMM2.
+// loaded once for both: the block pass's second product (CQR_GEMM_NPAIR=0: never).
 int npair_level() {
   static const int env = [] {
     const char* e = getenv("CQR_GEMM_NPAIR");
@@ -967,6 +1067,7 @@ TcGemm* tc_create(int mode, int64_t M, int64_t N, int64_t n, int64_t b, float* Q
   const uint32_t KE = (uint32_t)t->KE;
   bool ok = true;
   ok &= encode_2d(&t->tm_q_b, Q, kTF32, (uint64_t)M, (uint64_t)N, (uint64_t)ldq * 4, 32, BN);
+  ok &= encode_2d(&t->tm_q_c, Q, kTF32, (uint64_t)M, (uint64_t)N, (uint64_t)ldq * 4, 32, 32);
   for (int u = 0; u < 2; ++u) {
     ok &= encode_2d(&t->tm_ak[u][0], t->Ak_hi[u], kd, (uint64_t)M, (uint64_t)akc, (uint64_t)t->ldk * pe, KE, BM);
     ok &= encode_2d(&t->tm_ak[u][1], t->Ak_lo[u], kd, (uint64_t)M, (uint64_t)akc, (uint64_t)t->ldk * pe, KE, BM);
@@ -1172,12 +1273,17 @@ cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, in
   job.ldo = t->ldq;
   job.split_stride = 0;
   job.status = t->status;
-  maps.c = t->tm_q_b;
-  job.prefetch_c = 1;
   job.c_col0 = j0;
   job.oconst = q_inv(t);
   job.oinv = inv_of(t, j0);
-  job.pair_n = npair_level() >= 2 ? 1 : 0;
+  if (t->kind == kF16) {
+    maps.c = t->tm_q_c;
+    return launch_gemm<kF16, false, 2, 2, 2, 1, 1, true>(
+        maps, job, max_ctas > 0 ? std::min(max_ctas, t->num_sms) : t->num_sms, st,
+        t->pdl && st == t->pdl_st);
+  }
+  maps.c = t->tm_q_b;
+  job.prefetch_c = 1;
   return launch_mode(t, false, maps, job, st, max_ctas);
 }
 
