@@ -27,6 +27,15 @@ constexpr int kNT = 512;
 constexpr int kNW = kNT / 32;
 constexpr size_t kSmemCap = 227 * 1024;
 constexpr int kMaxOuter = 12, kMaxInner = 80;
+// Ends, as squares: of the refinement (|r| over |z|) and of one correction (over its |r|).  With
+// FP64 results 1e-15 and three or four corrections of 1e-5; with FP32 results 1e-11, where the
+// error of w is at most the condition number times that, a hundredth of the rounding of w to FP32
+// for a condition number of 60, and two corrections of 1.7e-6 reach it.
+template <typename T>
+struct Ends {
+  static constexpr double kOuter = sizeof(T) == 8 ? 1e-30 : 1e-22;
+  static constexpr float kInner = sizeof(T) == 8 ? 1e-10f : 3e-12f;
+};
 constexpr unsigned kTags = kMaxOuter * (kMaxInner + 1) + 8;
 // CTAs for e entries of Q_2: one per kFew entries up to kGroup CTAs (an exchange costs about
 // 2 us, a CTA's pass over 32,000 entries 3.7), then no more until each has kMany (problems on
@@ -297,7 +306,7 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
     }
     const double rr64 = block_sum(loc, bs);
     if (o == 0) zz = rr64;
-    if (!(rr64 > 1e-30 * zz) || (o > 0 && !(rr64 < 0.25 * prev))) break;
+    if (!(rr64 > Ends<T>::kOuter * zz) || (o > 0 && !(rr64 < 0.25 * prev))) break;
     prev = rr64;
     const double rn = sqrt(rr64), irn = 1.0 / rn;
     for (int j = tid; j < n; j += kNT) {
@@ -309,7 +318,7 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
     __syncthreads();
     // d: the correction over |r| by conjugate gradients in FP32
     float rr = 1.f;
-    for (int it = 0; it < kMaxInner && rr > 1e-10f; ++it) {
+    for (int it = 0; it < kMaxInner && rr > Ends<T>::kInner; ++it) {
       gram_vec<float, T>(S, Q2, ldq, rows, ns, n, in_smem != 0, p, reinterpret_cast<float*>(t),
                          reinterpret_cast<float*>(tp), Wf);
       ok = exchange<float, kNT>(xc, Wf, n, reinterpret_cast<float*>(red));
