@@ -132,8 +132,13 @@ cqr_status push_widths(cqr_batched bh) {
 cqr_status enqueue_encode(cqr_batched bh) {
   BK(cudaMemsetAsync(bh->d_R0, 0, bh->r_bytes, bh->st));
   BK(cudaMemsetAsync(bh->d_status, 0, sizeof(int) * 4 * bh->count, bh->st));
+  int both = 0;
+  for (const Geo& g : bh->geo) {
+    if (!g.protect_r) { both = 0; break; }
+    both = std::max(both, g.p_c);
+  }
   BK(launch_b_encode<float>(bh->d_inst, bh->count, bh->d_off_v, bh->tot_v, bh->d_off_h, bh->tot_h,
-                            bh->d_Gt_t, bh->d_Gh_t, bh->cfg.f, bh->st));
+                            bh->d_Gt_t, bh->d_Gh_t, bh->cfg.f, both, bh->st));
   return CQR_OK;
 }
 
