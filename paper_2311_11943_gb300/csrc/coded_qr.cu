@@ -1418,8 +1418,10 @@ namespace {
 
 cqr_status adj_scratch(cqr_handle h, size_t bytes) {
   if (h->adj_bytes >= bytes) return CQR_OK;
-  CK(cudaStreamSynchronize(h->st));
-  if (h->adj) cudaFree(h->adj);
+  if (h->adj) {  // work on the smaller one may be in flight
+    CK(cudaStreamSynchronize(h->st));
+    cudaFree(h->adj);
+  }
   h->adj = nullptr;
   h->adj_bytes = 0;
   if (cudaMalloc(&h->adj, bytes) != cudaSuccess) {
