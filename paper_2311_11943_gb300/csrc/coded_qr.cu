@@ -1531,7 +1531,7 @@ cqr_status adjoint_qr_t(cqr_handle h, const T* Q, int64_t ldq, const T* Qbar, in
       }
     }
   }
-  if (!solved) CK(launch_trsm_right<T>(1, R, g.ldr, n, Bb, 1, mp, mp, h->st));
+  if (!solved) CK(launch_trsm_right<T>(R, g.ldr, n, Bb, mp, mp, h->st));
   // Abar += G_0^T Bbar (G_0 is symmetric: its leading block I - V V^T / 2 is), rows < m
   if (g.f > 0) CK(launch_post_orth<T>(g, ptr<T>(h->B.Gt_t), Bb, mp, mp, n, Bb, mp, h->st));
   CK(launch_axpy2d<T>(g.m, n, T(1), Bb, 1, mp, Abar, 1, ldab, false, h->st));

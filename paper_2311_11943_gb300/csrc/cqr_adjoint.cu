@@ -110,18 +110,17 @@ __global__ void k_axpy2d(int64_t rows, int64_t cols, T alpha, const T* __restric
   }
 }
 
-// X op(R) = B in place (X overwrites B), R upper triangular n x n (ld ldr), B m x n with
-// element (i, j) at B[i rs + j cs].  trans = 1: X R^T = B, columns solved from the last
-// (X[:, j] = (B[:, j] - sum_{k>j} X[:, k] R[j, k]) / R[j, j]); trans = 0: X R = B, columns
-// solved from the first (X[:, j] = (B[:, j] - sum_{k<j} X[:, k] R[k, j]) / R[j, j]).
+// X R^T = B in place (X overwrites B), R upper triangular n x n (ld ldr), B m x n column-major
+// (ld cs): columns solved from the last
+// (X[:, j] = (B[:, j] - sum_{k>j} X[:, k] R[j, k]) / R[j, j]).
 // One CTA per block of rb <= 32 rows, held in shared memory [rb][n + 1]; right-looking: once
 // column j is final, its contribution leaves every column still to be solved.  Thread t works
 // on row t % 32 and the columns congruent to t / 32 modulo 8 (all lanes of a warp read the
 // same coefficient of R).  Used for diagonal blocks and for a few right-hand sides.
 template <typename T>
-__global__ void __launch_bounds__(256) k_trsm_right(int trans, const T* __restrict__ R, int64_t ldr,
-                                                    int n, T* __restrict__ B, int64_t rs,
-                                                    int64_t cs, int64_t m, int rb) {
+__global__ void __launch_bounds__(256) k_trsm_right(const T* __restrict__ R, int64_t ldr,
+                                                    int n, T* __restrict__ B, int64_t cs,
+                                                    int64_t m, int rb) {
   extern __shared__ __align__(16) unsigned char trsm_raw[];
   T* X = reinterpret_cast<T*>(trsm_raw);  // [rb][n + 1]
   const int tid = threadIdx.x, ld = n + 1;
@@ -129,27 +128,22 @@ __global__ void __launch_bounds__(256) k_trsm_right(int trans, const T* __restri
   const int nrow = (int)((m - r0) < rb ? (m - r0) : rb);
   for (int e = tid; e < nrow * n; e += 256) {
     const int j = e / nrow, r = e % nrow;
-    X[r * ld + j] = B[(r0 + r) * rs + (int64_t)j * cs];
+    X[r * ld + j] = B[r0 + r + (int64_t)j * cs];
   }
   __syncthreads();
   const int r = tid & 31, grp = tid >> 5;
-  for (int s = 0; s < n; ++s) {
-    const int j = trans ? n - 1 - s : s;
+  for (int j = n - 1; j >= 0; --j) {
     if (tid < nrow) X[tid * ld + j] /= R[j + (int64_t)j * ldr];
     __syncthreads();
     if (r < nrow) {
       const T xj = X[r * ld + j];
-      if (trans) {
-        for (int k = grp; k < j; k += 8) X[r * ld + k] -= xj * R[k + (int64_t)j * ldr];
-      } else {
-        for (int k = j + 1 + grp; k < n; k += 8) X[r * ld + k] -= xj * R[j + (int64_t)k * ldr];
-      }
+      for (int k = grp; k < j; k += 8) X[r * ld + k] -= xj * R[k + (int64_t)j * ldr];
     }
     __syncthreads();
   }
   for (int e = tid; e < nrow * n; e += 256) {
     const int j = e / nrow, r2 = e % nrow;
-    B[(r0 + r2) * rs + (int64_t)j * cs] = X[r2 * ld + j];
+    B[r0 + r2 + (int64_t)j * cs] = X[r2 * ld + j];
   }
 }
 
@@ -298,8 +292,8 @@ __global__ void __launch_bounds__(kIB) k_tri_inverse(const T* __restrict__ R, in
 }
 
 template <typename T>
-cudaError_t trsm_unblocked(int trans, const T* R, int64_t ldr, int n, T* B, int64_t rs, int64_t cs,
-                           int64_t m, cudaStream_t st) {
+cudaError_t trsm_unblocked(const T* R, int64_t ldr, int n, T* B, int64_t cs, int64_t m,
+                           cudaStream_t st) {
   const size_t cap = 200 * 1024;
   int rb = (int)std::min<int64_t>(32, (int64_t)(cap / ((size_t)(n + 1) * sizeof(T))));
   if (rb < 1) return cudaErrorInvalidValue;  // n too large for one row in shared memory
@@ -308,7 +302,7 @@ cudaError_t trsm_unblocked(int trans, const T* R, int64_t ldr, int n, T* B, int6
                                        (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)((m + rb - 1) / rb);
-  k_trsm_right<T><<<grid, 256, smem, st>>>(trans, R, ldr, n, B, rs, cs, m, rb);
+  k_trsm_right<T><<<grid, 256, smem, st>>>(R, ldr, n, B, cs, m, rb);
   return cudaGetLastError();
 }
 
@@ -346,31 +340,19 @@ cudaError_t launch_axpy2d(int64_t rows, int64_t cols, T alpha, const T* X, int64
   return cudaGetLastError();
 }
 
-// Blocked for a column-major B (rs == 1) with many rows: diagonal blocks of kTB columns are
-// solved by the row-block kernel, the rest of each step is one GEMM update
-//   trans = 1 (blocks from the last):  B[:, K] -= X[:, J] R[K, J]^T  for the blocks K < J
-//   trans = 0 (blocks from the first): B[:, K] -= X[:, J] R[J, K]    for the blocks K > J.
+// Blocked: diagonal blocks of kTB columns, from the last, are solved by the row-block kernel, the
+// rest of each step is one GEMM update, B[:, K] -= X[:, J] R[K, J]^T for the blocks K < J.
 template <typename T>
-cudaError_t launch_trsm_right(int trans, const T* R, int64_t ldr, int64_t n, T* B, int64_t rs,
-                              int64_t cs, int64_t m, cudaStream_t st) {
+cudaError_t launch_trsm_right(const T* R, int64_t ldr, int64_t n, T* B, int64_t cs, int64_t m,
+                              cudaStream_t st) {
   if (m <= 0 || n <= 0) return cudaSuccess;
   constexpr int kTB = 64;
-  // blocked when B is column-major (or a single contiguous row, cs == 1)
-  const bool colmajor = (rs == 1) || (m == 1);
-  if (!colmajor || n <= kTB) return trsm_unblocked<T>(trans, R, ldr, (int)n, B, rs, cs, m, st);
-  const int64_t nblk = (n + kTB - 1) / kTB;
-  for (int64_t s = 0; s < nblk; ++s) {
-    const int64_t J = trans ? nblk - 1 - s : s;
+  for (int64_t J = (n + kTB - 1) / kTB - 1; J >= 0; --J) {
     const int64_t j0 = J * kTB, jb = std::min<int64_t>(kTB, n - j0);
-    cudaError_t e = trsm_unblocked<T>(trans, R + j0 + j0 * ldr, ldr, (int)jb, B + j0 * cs, 1, cs, m, st);
-    if (e != cudaSuccess) return e;
-    if (trans && j0 > 0) {
-      e = launch_gemm_general<T>(0, 1, m, j0, jb, T(-1), B + j0 * cs, cs, R + j0 * ldr, ldr, T(1),
-                                 B, cs, st);
-    } else if (!trans && j0 + jb < n) {
-      e = launch_gemm_general<T>(0, 0, m, n - j0 - jb, jb, T(-1), B + j0 * cs, cs,
-                                 R + j0 + (j0 + jb) * ldr, ldr, T(1), B + (j0 + jb) * cs, cs, st);
-    }
+    cudaError_t e = trsm_unblocked<T>(R + j0 + j0 * ldr, ldr, (int)jb, B + j0 * cs, cs, m, st);
+    if (e == cudaSuccess && j0 > 0)
+      e = launch_gemm_general<T>(0, 1, m, j0, jb, T(-1), B + j0 * cs, cs, R + j0 * ldr, ldr, T(1), B, cs,
+                                 st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -422,8 +404,8 @@ cudaError_t bounds_take_adjoint(int* code, int* site) { return bounds_take_here(
                                        cudaStream_t);                                            \
   template cudaError_t launch_axpy2d<T>(int64_t, int64_t, T, const T*, int64_t, int64_t, T*,     \
                                         int64_t, int64_t, bool, cudaStream_t);                   \
-  template cudaError_t launch_trsm_right<T>(int, const T*, int64_t, int64_t, T*, int64_t,        \
-                                            int64_t, int64_t, cudaStream_t);
+  template cudaError_t launch_trsm_right<T>(const T*, int64_t, int64_t, T*, int64_t, int64_t,    \
+                                            cudaStream_t);
 
 CQR_ADJ_INSTANTIATE(float)
 CQR_ADJ_INSTANTIATE(double)

@@ -213,10 +213,10 @@ cudaError_t launch_copyltu(const T* Mm, int64_t n, T* S, cudaStream_t st);
 template <typename T>
 cudaError_t launch_axpy2d(int64_t rows, int64_t cols, T alpha, const T* X, int64_t xrs, int64_t xcs,
                           T* Y, int64_t yrs, int64_t ycs, bool overwrite, cudaStream_t st);
-// X op(R) = B in place, R n x n upper; trans = 1: X R^T = B; trans = 0: X R = B.
+// X R^T = B in place, R n x n upper, B m x n column-major (ld cs).
 template <typename T>
-cudaError_t launch_trsm_right(int trans, const T* R, int64_t ldr, int64_t n, T* B, int64_t rs,
-                              int64_t cs, int64_t m, cudaStream_t st);
+cudaError_t launch_trsm_right(const T* R, int64_t ldr, int64_t n, T* B, int64_t cs, int64_t m,
+                              cudaStream_t st);
 
 // R^T x = b in place for R upper triangular, k right-hand sides.
 template <typename T>
