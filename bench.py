@@ -62,11 +62,9 @@ MODES = {"f64": ("f64", "simt"), "f32": ("f32", "simt"), "tf32": ("f32", "tf32")
          "3xtf32": ("f32", "3xtf32"), "bf16": ("f32", "bf16"), "bf16x3": ("f32", "bf16x3")}
 L2_BYTES = 126 * 1024 * 1024
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a dominant kernel from
-# one ncu capture of the current kernel, keyed by (config, mode, profile class):
-# profiles/k_panel_c3.md for the 20480 x 256 panel of the 16384^2 workload (captured on a
-# 16384 x 8192 problem with the same panel shape and grid).  Absent (the 4096^2 register panel
-# has changed since its capture): reported as null.
-NCU_TRAFFIC = {("c3", "3xtf32", "panel_icgs"): 21.079552e6 + 0.007680e6}
+# one ncu capture of the current kernel, keyed by (config, mode, profile class).  Absent (the
+# panel and update kernels have changed since their captures): reported as null.
+NCU_TRAFFIC = {}
 
 
 def coded_flops(m, n, p_r, p_c, f, b, protect_r=True):
@@ -724,7 +722,11 @@ def roofline(args, cfg, prof, geo, dtype, mma, es, peaks_here):
         algo = per_step[dom_name] * args.steps / dom_launches
         achieved = algo / (dom_ms / dom_launches * 1e-3) / 1e12
         tf32 = (peaks_here or {}).get("tf32_tflops_sustained")
-        if dtype == "f64":
+        if dtype == "f64" and dom_name in ("tc_update", "tc_rbar"):
+            peak = peaks["bf16_tflops_sustained"] / 28.0
+            rl = {"bound": "tensor", "unit": "TFLOP/s", "peak_source": "%s bf16 sustained / 28 (digit "
+                  "products per FP64 product)" % peak_src}
+        elif dtype == "f64":
             fp64 = (peaks_here or {}).get("fp64_tflops")
             peak = fp64 or 152 * 2 * 2 * 2.07e9 / 1e12
             rl = {"bound": "alu", "unit": "TFLOP/s", "peak_source":
@@ -734,22 +736,16 @@ def roofline(args, cfg, prof, geo, dtype, mma, es, peaks_here):
             peak = 152 * 128 * 2 * 2.07e9 / 1e12
             rl = {"bound": "alu", "unit": "TFLOP/s", "peak_source": "FP32 CUDA-core: 152 SMs x "
                   "128 FFMA/clk x 2 flop x 2.07 GHz"}
-        elif mma in ("bf16", "bf16x3"):
-            k = 3.0 if mma == "bf16x3" else 1.0
+        elif mma != "tf32":  # 3xtf32: FP16 halves, at the BF16 rate
+            k = 1.0 if mma == "bf16" else 3.0
             peak = peaks["bf16_tflops_sustained"] / k
             rl = {"bound": "tensor", "unit": "TFLOP/s", "peak_source": "%s bf16 sustained%s"
-                  % (peak_src, " / 3 (three bf16 MMAs per FP32-accurate product)" if k > 1 else "")}
+                  % (peak_src, " / 3 (three 16-bit MMAs per FP32-accurate product)" if k > 1 else "")}
         else:
-            k = 3.0 if mma == "3xtf32" else 1.0
-            if tf32:
-                peak = tf32 / k
-                src = "tf32 sustained measured in this run"
-            else:
-                peak = peaks["bf16_tflops_sustained"] * 1.1 / 2.25 / k
-                src = "%s bf16 sustained x nominal tf32/bf16 ratio 1.1/2.25" % peak_src
-            rl = {"bound": "tensor", "unit": "TFLOP/s", "peak_source": src + (
-                  " / 3 (three tf32 MMAs per FP32-accurate product)" if k > 1 else "")}
-            rl["tensor_pipe_frac"] = achieved * k / (peak * k)
+            peak = tf32 or peaks["bf16_tflops_sustained"] * 1.1 / 2.25
+            rl = {"bound": "tensor", "unit": "TFLOP/s", "peak_source":
+                  "tf32 sustained measured in this run" if tf32 else
+                  "%s bf16 sustained x nominal tf32/bf16 ratio 1.1/2.25" % peak_src}
         rl.update(achieved=achieved, peak=peak, frac=achieved / peak)
     else:
         algo = panel_bytes * args.steps / dom_launches if dom_name == "panel_icgs" else None

@@ -179,15 +179,17 @@ cqr_status coded_qr_encode(cqr_handle h, const void* A, int64_t lda);
  * panel_begin must equal the next unfactored panel; panel_end = -1 means the last panel.
  * Returns CQR_ESTATE while erasures are pending (erased tiles hold NaN).
  *
- * Scheduling (FP32 tensor-core handles whose panel runs on one thread-block cluster): the
- * trailing update of each panel is split into the next panel's columns, on an internal
- * stream of the highest priority, and the rest, on an internal stream of the lowest
- * priority that overlaps the next panel's factorisation; kernels on the first stream use
- * programmatic dependent launch.  Both streams fork from and join into cfg.stream inside the
- * call.  Environment switches, for comparisons only: CQR_LOOKAHEAD=0 (one stream, no
- * split), CQR_PDL=0 (no programmatic dependent launch), CQR_PANEL_REG=0 (no register-
- * resident panel kernel), CQR_PANEL_CLUSTER=0 (no single-cluster panel kernels),
- * CQR_PANEL_RPL=r (rows per lane of the shared-memory / grid panel kernels). */
+ * Scheduling: the launches follow one another on cfg.stream; on FP32 tensor-core handles they use
+ * programmatic dependent launch.  ICGS and MGS panels run in sub-blocks of 16 columns, a
+ * cooperative launch over as many CTAs as hold the rows.  Where the panel does not fit that kernel
+ * (or with CQR_PANEL_BLK=0) it goes column by column; if it then runs on one thread-block cluster
+ * of an FP32 tensor-core handle, the trailing update of each panel is split into the next panel's
+ * columns, on an internal stream of the highest priority, and the rest, on one of the lowest
+ * priority that overlaps the next panel's factorisation; both fork from and join into cfg.stream
+ * inside the call.  Environment switches, for comparisons only: CQR_PANEL_BLK=0 (column by
+ * column), CQR_LOOKAHEAD=0 (one stream, no split), CQR_PDL=0 (no programmatic dependent launch),
+ * CQR_PANEL_REG=0 (no register-resident panel kernel), CQR_PANEL_CLUSTER=0 (no single-cluster
+ * panel kernels), CQR_PANEL_RPL=r (rows per lane of the shared-memory / grid panel kernels). */
 cqr_status coded_qr_factor(cqr_handle h, int32_t panel_begin, int32_t panel_end);
 
 /* a6.  Fail-stop erasure of nodes (Section 2 "Failure model"): tiles (host) holds `count`
@@ -297,8 +299,8 @@ cqr_status coded_qr_debug_bounds_selftest(void* stream);
  * Appendix A's Algorithm CGS (right-looking, with the ICGS criterion) performs one reduction
  * across its CTAs per column; with everything else on chip, those reductions bound how fast a
  * column can go.  This call runs the reductions of one M x bk FP32 panel -- a first one of
- * 2 bk entries, then bk - 1 - j entries for column j -- with the panel kernel's own exchange
- * code, launch shape and shared-memory footprint but no column arithmetic, `reps` times in one
+ * 2 bk entries, then bk - 1 - j entries for column j -- with the exchange code, launch shape and
+ * shared-memory footprint of the column-by-column panel kernels but no column arithmetic, `reps` times in one
  * launch after a one-launch warm-up, and stores the mean device time per panel column in
  * microseconds (CUDA events on `stream`; the call synchronises the stream).
  *   kind 0: the register panel (one cluster; bk <= 128 and M within its registers);
@@ -429,8 +431,9 @@ cqr_status coded_qr_batched_sync_status(cqr_batched bh, int32_t* first_bad, int6
 /* Phase clocks of the persistent factor launch (instrumentation, no counterpart in the paper).
  * With enable != 0 every later factor launch of the batch (direct, or recorded into a new
  * graph) adds, for each CTA, the SM clock cycles it spent in each phase to counters of the
- * batch (allocated on the first enable): in-launch recovery, panel, the product Qbar^T B,
- * its reduction into Rbar, the update B -= Qbar Rbar, the rest (work queue, the wait at the
+ * batch (allocated on the first enable): in-launch recovery, panel, the product Qbar^T B
+ * (the panel's own streamed products included),
+ * its reduction into Rbar, the update B -= Qbar Rbar (the panel's too), the rest (work queue, the wait at the
  * end), and the parts of the two products spent at the top of each pipeline stage waiting for
  * its copies and the CTA barrier.  Thread 0 of the CTA reads the clock at the phase
  * boundaries, so the cost when on is a few instructions per pipeline stage; when off, one
@@ -460,8 +463,8 @@ cqr_status coded_qr_adjoint_qr(cqr_handle h, const void* Q, int64_t ldq, const v
                                int64_t ldab);
 /* coded_qr_adjoint_lstsq: x = argmin |A x - y| (x n x nrhs from coded_qr_solve on this handle,
  * A m x n with full column rank, y m x nrhs).  With z = (A^T A)^{-1} xbar evaluated through the
- * coded factors as R^{-1} (I - Q_2^T Q_2)^{-1} R^{-T} xbar (FP64 conjugate gradients for the
- * middle factor) and r = y - A x:  Abar += r z^T - (A z) x^T,  ybar += A z.  Abar or ybar may
+ * coded factors as R^{-1} (I - Q_2^T Q_2)^{-1} R^{-T} xbar (the middle factor by refinement
+ * with FP64 residuals, or FP64 conjugate gradients for very long rows) and r = y - A x:  Abar += r z^T - (A z) x^T,  ybar += A z.  Abar or ybar may
  * be NULL.  Needs Q_1 in the handle (CQR_ESTATE after an in-place post-orthogonalisation). */
 cqr_status coded_qr_adjoint_lstsq(cqr_handle h, const void* A, int64_t lda, const void* y,
                                   int64_t ldy, const void* x, int64_t ldx, const void* xbar,

@@ -11,8 +11,8 @@ outputs, coded_qr_adjoint_lstsq for x).  Only tall problems (m > n) are accepted
 ones the solve post-orthogonalises in place and the least-squares adjoint needs Q_1.
 
 The problems of a batch run concurrently, each on its own CUDA stream (joined to the caller's
-stream at the end): one problem's panel factorisation occupies at most one thread-block
-cluster, so several of them share the GPU.
+stream at the end): one problem's panel factorisation takes a CTA per 128 or more
+rows, so several of them share the GPU.
 """
 import torch
 

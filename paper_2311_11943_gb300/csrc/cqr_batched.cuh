@@ -11,9 +11,10 @@ constexpr int kBMax = 64;  // widest panel of the batched kernel
 constexpr int kWC = 64;    // trailing columns per update chunk
 
 // Phases of the factor launch's clocks (BFactorLaunch::prof): in-launch recovery; the panel
-// (ICGS column steps, the slice's copies); the product S = Qbar^T B; its reduction into Rbar
-// (K-split sum, cluster sum, store into R); the update B -= Qbar Rbar; everything else (the
-// work queue, the wait at the end); and, split off the two products, the time spent at the
+// (its Cholesky factors and column steps); the product S = Qbar^T B, the panel's own products
+// included; its reduction into Rbar (K-split sum, cluster sum, store into R); the update
+// B -= Qbar Rbar, the panel's own included; everything else (the work queue, the wait at the
+// end); and, split off the two products, the time spent at the
 // top of each pipeline stage waiting for its copies and for the CTA's barrier.
 // prof[kPhases] counts the CTAs that added their clocks.
 enum { PH_RECOVER = 0, PH_PANEL, PH_SPROD, PH_RBAR, PH_UPDATE, PH_OTHER, PH_SPROD_WAIT,
