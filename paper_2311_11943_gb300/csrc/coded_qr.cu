@@ -852,17 +852,21 @@ cqr_status post_orth_y(cqr_handle h, const T* y, int64_t ldy, int32_t nrhs, T* y
 }
 
 // ------------------------------------------------------------------------------- solve
-// w = (I - Q_2^T Q_2)^{-1} Q_1^T y (or ... u) into w: by iterative refinement where its vectors
+// w = (I - Q_2^T Q_2)^{-1} Q_1^T y (or ... u), k right-hand sides: by iterative refinement where its vectors
 // fit shared memory (n up to about 7000), else by conjugate gradients in FP64.
 template <typename T>
-cudaError_t ls_middle(cqr_handle h, const T* y, const T* u, T* w) {
+cudaError_t ls_middle(cqr_handle h, int k, const T* y, int64_t ldy, const T* u, int64_t ldu, T* w,
+                      int64_t ldw) {
   const Geo& g = h->g;
   bool taken = false;
-  const cudaError_t e = launch_ls_refine<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y, u, w,
-                                            h->B.cg, h->B.lsx, h->B.status, h->num_sms, h->st, &taken);
+  cudaError_t e = launch_ls_refine<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, k, y, ldy, u, ldu,
+                                      w, ldw, h->B.cg, h->B.lsx, h->B.status, h->num_sms, h->st, &taken);
   if (taken || e != cudaSuccess) return e;
-  return launch_ls_cg<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y, w, h->B.cg, h->B.bar,
-                         h->B.status, h->num_sms, h->st, u);
+  for (int j = 0; j < k && e == cudaSuccess; ++j)
+    e = launch_ls_cg<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y ? y + j * ldy : nullptr,
+                        w + j * ldw, h->B.cg, h->B.bar, h->B.status, h->num_sms, h->st,
+                        u ? u + j * ldu : nullptr);
+  return e;
 }
 
 template <typename T>
@@ -870,13 +874,11 @@ cqr_status solve_t(cqr_handle h, const T* y, int64_t ldy, T* x, int64_t ldx, int
   const Geo& g = h->g;
   const bool square = (g.m == g.n && g.m_pad == g.m);
   if (!square) {
-    // least squares through A = Q_1 R: CG in FP64 on (I - Q_2^T Q_2) w = Q_1^T y, then R x = w
+    // least squares through A = Q_1 R: (I - Q_2^T Q_2) w = Q_1^T y, then R x = w
     if (h->postorth_inplace) return CQR_ESTATE;  // Q_1 was overwritten by G_0 Q_1
-    for (int32_t k = 0; k < nrhs; ++k) {
-      {
-        ProfScope ps(h, K_SOLVE_GEMV, 1);
-        CK(ls_middle<T>(h, y + (int64_t)k * ldy, nullptr, x + (int64_t)k * ldx));
-      }
+    {
+      ProfScope ps(h, K_SOLVE_GEMV, nrhs);
+      CK(ls_middle<T>(h, nrhs, y, ldy, nullptr, 0, x, ldx));
     }
     ProfScope ps(h, K_TRSV, nrhs);
     CK(launch_trsv_upper<T>(ptr<T>(h->B.R), g.ldr, g.n, x, ldx, nrhs, h->st));
@@ -1554,9 +1556,8 @@ cqr_status adjoint_lstsq_t(cqr_handle h, const T* A, int64_t lda, const T* y, in
   // u = R^{-T} xbar: rows of the (k x n) view solve u^T R = xbar^T
   CK(launch_axpy2d<T>(n, k, T(1), xbar, 1, ldxb, u, 1, n, true, h->st));
   CK(launch_trsv_upper_t<T>(R, g.ldr, n, u, n, k, h->st));
-  // w = (I - Q_2^T Q_2)^{-1} u (FP64 conjugate gradients), z = R^{-1} w
-  for (int32_t j = 0; j < k; ++j)
-    CK(ls_middle<T>(h, nullptr, u + (size_t)j * n, w + (size_t)j * n));
+  // w = (I - Q_2^T Q_2)^{-1} u, z = R^{-1} w
+  CK(ls_middle<T>(h, k, nullptr, 0, u, n, w, n));
   CK(launch_trsv_upper<T>(R, g.ldr, n, w, n, k, h->st));
   const T* z = w;
   // Az, r = y - A x

@@ -192,13 +192,14 @@ cudaError_t launch_ls_cg(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, int6
                          cudaStream_t st, const T* u = nullptr);
 
 // The same by iterative refinement (cqr_lstsq.cu); *taken false (nothing launched) when its
-// vectors do not fit shared memory.  z: n doubles of workspace; xws: ls_refine_bytes of device
-// memory, zero before the first launch and kept between launches.
+// vectors do not fit shared memory.  k right-hand sides; z: min(k, 4) n doubles of workspace; xws:
+// ls_refine_bytes of device memory, zero before the first launch and kept between launches.
 size_t ls_refine_bytes(int64_t n, int num_sms);
 template <typename T>
 cudaError_t launch_ls_refine(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, int64_t c, int64_t n,
-                             const T* y, const T* u, T* x, double* z, void* xws, int* status,
-                             int num_sms, cudaStream_t st, bool* taken);
+                             int k, const T* y, int64_t ldy, const T* u, int64_t ldu, T* x,
+                             int64_t ldx, double* z, void* xws, int* status, int num_sms,
+                             cudaStream_t st, bool* taken);
 
 // ---------------------------------------------------------------- adjoint building blocks
 // C (M x N) = alpha op(A) op(B) + beta C (op = transpose when ta / tb); beta == 0 ignores C.
