@@ -3,15 +3,15 @@
 // the coded Q.  SPD with condition number at most 1 + ||G~||^2, a property of the code.
 //
 // Iterative refinement: the residual r = z - w + Q_2^T (Q_2 w) and w in FP64, the corrections by
-// conjugate gradients in FP32 to five digits, until |r| <= 1e-15 |z| (the accuracy of conjugate
-// gradients in FP64 throughout) or no longer falling.  Three or four FP64 residuals instead of
-// some ninety FP64 iterations: the FP64 pipes give about two products per cycle and SM, the
+// conjugate gradients in FP32 to five or six digits, until |r| <= 1e-15 |z| (the accuracy of
+// conjugate gradients in FP64 throughout; 1e-11 where the result is FP32, see Ends) or no longer
+// falling.  Two to four FP64 residuals instead of some ninety FP64 iterations: the FP64 pipes give about two products per cycle and SM, the
 // FP32 ones 128, and an iteration is then one pass over Q_2 and one sum over the CTAs.
 // G CTAs each hold rows of Q_2 in shared memory (transposed while they are loaded, so that both
 // products read along rows), every vector of n entries is held by every CTA, and the n sums of
 // Q_2^T t go through cqr_exchange.cuh: one exchange per iteration instead of four grid
 // barriers, and no traffic for Q_2.  Measured, FP64 iterations on 32 CTAs before, this after
-// (FP32, one right-hand side): Q_2 2048 x 2048 12.3 and 0.96 ms, 1538 x 1320 3.5 and 0.49 ms.
+// (FP32, one right-hand side): Q_2 2048 x 2048 12.3 and 0.73 ms, 1538 x 1320 3.5 and 0.36 ms.
 #include <math.h>
 
 #include <algorithm>
