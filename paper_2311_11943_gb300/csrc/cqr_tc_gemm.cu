@@ -585,7 +585,10 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
 // Ak_hi / Ak_lo; for GEMM2's A (row-major, row stride bkp): At_hi / At_lo; columns k >= bk
 // zero-filled up to bkp (and up to 128 columns for GEMM1's M tile).  With Qr != nullptr the
 // finished panel is also copied into the row-major planes of all computed columns
-// (Qr[r * ldrow + kb + k]), the K-major operand of the block reorthogonalisation.
+// (Qr[r * ldrow + kb + k]), the K-major operand of the block reorthogonalisation; columns
+// bk .. qcols - 1 of that copy are zero: a later product reads whole stages of K, the columns behind
+// the last computed one against zero rows, and what an earlier factorisation left there need
+// not be finite.
 // Operand planes: x = hi + lo with hi = rna_tf32(x) (TF32; hi = x with one product, the MMA
 // reads TF32 from the FP32 word) or hi = rn(x), lo = rn(x - hi) in BF16 or FP16 (there x is
 // scaled: by cscale[k] where given, else by scale).
@@ -612,7 +615,7 @@ __global__ void __launch_bounds__(256) k_split_panel(const float* __restrict__ Q
                                                      P* __restrict__ Ak_lo, int64_t ldk,
                                                      P* __restrict__ At_hi, P* __restrict__ At_lo,
                                                      P* __restrict__ Qr_hi, P* __restrict__ Qr_lo,
-                                                     int64_t ldrow, int64_t kb, float scale,
+                                                     int64_t ldrow, int64_t kb, int qcols, float scale,
                                                      const float* __restrict__ cscale) {
   __shared__ P sh[32][33], sl[32][33];
   pdl_wait();
@@ -645,7 +648,7 @@ __global__ void __launch_bounds__(256) k_split_panel(const float* __restrict__ Q
       At_hi[rr * bkp + k] = h;
       if (nplanes == 2) At_lo[rr * bkp + k] = l;
     }
-    if (Qr_hi && k < bk) {
+    if (Qr_hi && k < qcols) {
       Qr_hi[rr * ldrow + kb + k] = h;
       if (nplanes == 2) Qr_lo[rr * ldrow + kb + k] = l;
     }
@@ -1050,13 +1053,6 @@ TcGemm* tc_create(int mode, int64_t M, int64_t N, int64_t n, int64_t b, float* Q
     t->Qr_lo = take((size_t)M * t->ldrow * pe);
     t->Sh = take((size_t)t->ldrow * akc * pe);
     t->Sl = take((size_t)t->ldrow * akc * pe);
-    // columns not yet computed are read (times zero rows of S) when kb is not a multiple of
-    // the stage K: keep them finite
-    if (cudaMemsetAsync(t->Qr_hi, 0, (size_t)M * t->ldrow * pe, st) != cudaSuccess ||
-        cudaMemsetAsync(t->Qr_lo, 0, (size_t)M * t->ldrow * pe, st) != cudaSuccess) {
-      delete t;
-      return nullptr;
-    }
   }
   t->cs = t->ci = nullptr;
   if (t->kind == kF16) {
@@ -1144,8 +1140,9 @@ cudaError_t split_panel(TcGemm* t, int64_t kb, int bk, bool finished, const floa
                         cudaStream_t st) {
   const int bkp = (int)t->bkp;  // the planes' stride in the tensor maps, also for a narrower last panel
   const int m1 = (bk + BM - 1) / BM;
-  dim3 grd((unsigned)((t->M + 31) / 32), (unsigned)((std::max(bkp, m1 * BM) + 31) / 32));
   void* qh = finished ? t->Qr_hi : nullptr;
+  const int qcols = qh ? (int)(round_to(kb + bk, t->KE) - kb) : 0;  // to the end of a stage of K
+  dim3 grd((unsigned)((t->M + 31) / 32), (unsigned)((std::max({bkp, m1 * BM, qcols}) + 31) / 32));
   const bool pdl = t->pdl && st == t->pdl_st;
   const float* q0 = t->Q + kb * t->ldq;
   return with_plane(t, [&](auto tag) {
@@ -1153,7 +1150,7 @@ cudaError_t split_panel(TcGemm* t, int64_t kb, int bk, bool finished, const floa
     return launch_k(k_split_panel<P>, grd, dim3(256), 0, st, pdl, q0, t->ldq, t->M, bk, bkp,
                     (int)(m1 * BM), t->nplanes, pl<P>(t->Ak_hi[buf]), pl<P>(t->Ak_lo[buf]), t->ldk,
                     pl<P>(t->At_hi[buf]), pl<P>(t->At_lo[buf]), pl<P>(qh), pl<P>(t->Qr_lo), t->ldrow, kb,
-                    q_scale(t), cscale);
+                    qcols, q_scale(t), cscale);
   });
 }
 }  // namespace
@@ -1408,7 +1405,7 @@ cudaError_t tc_gemm_sub3(bool a_trans, const float* A, int64_t lda, const float*
     float* lo = hi + kp * M;
     const dim3 grd((unsigned)((K + 31) / 32), (unsigned)((M + 31) / 32));
     k_split_panel<float><<<grd, 256, 0, st>>>(A, lda, K, (int)M, 0, (int)M, 2, hi, lo, kp, nullptr,
-                                              nullptr, nullptr, nullptr, 0, 0, 1.f, nullptr);
+                                              nullptr, nullptr, nullptr, 0, 0, 0, 1.f, nullptr);
     ok &= encode_2d(&maps.a[0], hi, kTF32, (uint64_t)K, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
     ok &= encode_2d(&maps.a[1], lo, kTF32, (uint64_t)K, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
   } else {
@@ -1416,7 +1413,7 @@ cudaError_t tc_gemm_sub3(bool a_trans, const float* A, int64_t lda, const float*
     float* lo = hi + M * kp;
     const dim3 grd((unsigned)((M + 31) / 32), (unsigned)((kp + 31) / 32));
     k_split_panel<float><<<grd, 256, 0, st>>>(A, lda, M, (int)K, (int)kp, 0, 2, nullptr, nullptr, 0, hi,
-                                              lo, nullptr, nullptr, 0, 0, 1.f, nullptr);
+                                              lo, nullptr, nullptr, 0, 0, 0, 1.f, nullptr);
     ok &= encode_2d(&maps.a[0], hi, kTF32, (uint64_t)kp, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
     ok &= encode_2d(&maps.a[1], lo, kTF32, (uint64_t)kp, (uint64_t)M, (uint64_t)kp * 4, 32, BM);
   }
