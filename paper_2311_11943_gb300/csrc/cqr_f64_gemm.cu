@@ -494,9 +494,10 @@ struct F64Gemm {
   CUtensorMap mqc, mqr, mbt, mrb;
 };
 
-// Workspace of the handle (0: its updates are too small to gain, or too tall).
+// Workspace of the handle (0: its updates are too small to gain, or too tall, or the panel is wider
+// than one sum of the update's K may be).
 size_t f64_gemm_bytes(int64_t M, int64_t N, int64_t b) {
-  if (M > (int64_t)kMaxSplits * kMaxK || !f64_gemm_pays(M, N - b, b)) return 0;
+  if (M > (int64_t)kMaxSplits * kMaxK || b > kMaxK || !f64_gemm_pays(M, N - b, b)) return 0;
   const int64_t kpm = up64(M), kpb = up64(b), cols = col_block(M, N);
   return al256((size_t)b * kD * kpm * 2) + al256((size_t)M * kD * kpb * 2) +
          al256((size_t)cols * kD * kpm * 2) + al256((size_t)cols * kD * kpb * 2) +
@@ -547,6 +548,7 @@ int64_t f64_gemm_cols(const F64Gemm* t) { return t->cols; }
 namespace {
 cudaError_t launch_oz(const CUtensorMap& a, const CUtensorMap& b, const OzJob& job, int num_sms,
                       cudaStream_t st) {
+  if (job.kchunk > kMaxK) return cudaErrorInvalidValue;  // the sums would overflow
   cudaError_t e = cudaFuncSetAttribute((const void*)k_f64_gemm,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTotal);
   if (e != cudaSuccess) return e;
