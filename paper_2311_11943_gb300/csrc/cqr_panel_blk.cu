@@ -62,6 +62,33 @@ __device__ __forceinline__ float round_up_to<float>(double t) { return __double2
 template <>
 __device__ __forceinline__ double round_up_to<double>(double t) { return t; }
 
+// A squared norm as m 4^h, 1 <= m < 4 (h = 0 for floats, whose range holds it), and |x| 2^h as a
+// float (zero below its range, infinite above): the test of what a sub-block amplifies multiplies
+// entries of U^{-T} by column norms, whose product is a pure number also where neither fits a
+// float.  By integer operations on the high word, since the FP64 pipe is slow.
+__device__ __forceinline__ float norm_of(float v, int& h) {
+  h = 0;
+  return sqrtf(v);
+}
+__device__ __forceinline__ float norm_of(double v, int& h) {
+  const int hi = __double2hiint(v);
+  if (hi < 0x00100000 || hi >= 0x7ff00000) {  // no pivot comes of it
+    h = 0;
+    return 0.f;
+  }
+  const int ex = (hi >> 20) - 1023;
+  h = ex >> 1;
+  return sqrtf(__int_as_float(((127 + (ex & 1)) << 23) | ((hi & 0xfffff) << 3)));
+}
+__device__ __forceinline__ float scaled_abs(float x, int) { return fabsf(x); }
+__device__ __forceinline__ float scaled_abs(double x, int h) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  const int ex = (hi >> 20) - 1023 + 127 + h;
+  if (hi < 0x00100000 || ex <= 0) return 0.f;
+  return ex >= 255 || hi >= 0x7ff00000 ? __int_as_float(0x7f800000)
+                                       : __int_as_float((ex << 23) | ((hi & 0xfffff) << 3));
+}
+
 // 16 bytes of a column in shared memory and their arithmetic: four floats as two packed f32x2
 // pairs, or two doubles.
 __device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c) {
@@ -277,6 +304,7 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
   __shared__ __align__(16) T sU[S * S], sLi[S * S], sU2[S * S];
   __shared__ __align__(16) T sRow[16 * S], sD[S];
   __shared__ float sNrm[S];
+  __shared__ int sExp[S];
   __shared__ int sGood;
   __shared__ unsigned sFail;
   const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x;
@@ -400,12 +428,19 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
     } else if (warp == 0) {
       gd = cholesky<T>(second ? c.red : c.W, second ? S : w, nx, second ? sU2 : sU, sLi, sD, sRow);
       if (!second) {
-        if (lane < n) sNrm[lane] = sqrtf((float)c.W[lane * w + lane]);
+        if (lane < n) {
+          int h;
+          sNrm[lane] = norm_of(c.W[lane * w + lane], h);
+          sExp[lane] = h;
+        }
         __syncwarp();
         float amp = 0.f;
         if (lane < gd)
 #pragma unroll 4
-          for (int k = 0; k < S; ++k) amp += fabsf((float)sLi[lane * S + k]) * sNrm[min(k, n - 1)];
+          for (int k = 0; k < S; ++k) {
+            const int q = min(k, n - 1);
+            amp += scaled_abs(sLi[lane * S + k], sExp[q]) * sNrm[q];
+          }
         const unsigned bad = __ballot_sync(0xffffffffu, lane > 0 && lane < gd && !(amp <= kMaxAmp));
         if (bad) gd = min(gd, __ffs(bad) - 1);
         // the ICGS test, from the panel's second column on
