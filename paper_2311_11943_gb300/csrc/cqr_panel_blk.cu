@@ -16,12 +16,20 @@
 //   T = P_S U^{-1},  Z1 = Q[:, 0:j]^T T,  U2^T U2 = T^T T - Z1^T Z1,  Q_S = (T - Q[:, 0:j] Z1) U2^{-1},
 //   R[0:j, S] += Z1 U,  R[j:j+S, j:b] = U2 U and U2^{-T} U^{-T} W[:, S:].
 // The Cholesky form and the column recurrence differ by rounding of order u times the squared
-// condition number of the sub-block, so a sub-block is taken this way only up to its first
-// column whose pivot is not positive and finite or whose row of U^{-T} amplifies rounding by
-// more than kMaxAmp (the sum over k of |U^{-T}_ak| |p_k|, 1 for orthogonal columns).  That
-// column goes through the column recurrence itself (products, ICGS reorthogonalisation when the
-// test asks for it, normalisation, update), and the next sub-block starts behind it.  Every CTA
-// takes the same decisions from the same sums.
+// condition number of the sub-block.  Where a row of U^{-T} amplifies rounding by more than
+// kMaxAmp (the sum over k of |U^{-T}_ak| |p_k|, 1 for orthogonal columns; nearly dependent columns)
+// the sub-block always takes the second projection, and three things change so that no digit
+// depends on the first factor: T = P_S U^{-1} by substitution (P_S = T U to rounding), the
+// rows of R behind the sub-block from products with T (the second projection's products then
+// run over all columns), and a pivot below kFloor times its column's squared norm is raised to
+// that, which only scales its column of T.  A column whose second norm cannot be had this way either
+// (amplification above kMaxHard) or whose pivot is not positive and finite goes through the column
+// recurrence itself (products, ICGS reorthogonalisation when the test asks for it, normalisation,
+// update), and the next sub-block starts behind it.  Without the ICGS test (MGS) the second
+// projection is within the sub-block.  Every CTA takes the same decisions from the same sums.
+// Why not the recurrence for every column above kMaxAmp: 4096 x 2048, b = 128, every second column
+// within 1e-3 of the one before, 24.5 ms that way (8.4 ms by the column-by-column kernels), 4.8 ms
+// so; every seventh column 7.7 (5.8), 4.8 ms.
 //
 // Why: the panel is bound by the latency of its reductions and by passes over the slice.  Per
 // column, one exchange and one pass over the slice cost 2.2 us (5120 x 128, one cluster of 16)
@@ -51,6 +59,13 @@ constexpr size_t kSmemCap = 227 * 1024;
 // Cholesky: U = I + E / 2 on the diagonal and I + E above it, with E^2 below rounding.
 template <typename T>
 constexpr T kNearI = sizeof(T) == 4 ? T(1.0 / 8192) : T(1.0 / (1 << 27));
+// Largest amplification that the second projection mends (u kMaxHard^2 is at most 1/4: T stays well
+// conditioned), and the floor of a pivot over its column's squared norm (amplification about
+// 1 / sqrt(kFloor) then).
+template <typename T>
+constexpr float kMaxHard = sizeof(T) == 4 ? 2048.f : 16777216.f;
+template <typename T>
+constexpr T kFloor = sizeof(T) == 4 ? T(1.0 / (1 << 18)) : T(1.0 / (1ll << 44));
 // Row stride of the solved coefficients: 16-byte rows
 template <typename T>
 constexpr int kSY = kS<T> + 16 / (int)sizeof(T);
@@ -87,6 +102,21 @@ __device__ __forceinline__ float scaled_abs(double x, int h) {
   if (hi < 0x00100000 || ex <= 0) return 0.f;
   return ex >= 255 || hi >= 0x7ff00000 ? __int_as_float(0x7f800000)
                                        : __int_as_float((ex << 23) | ((hi & 0xfffff) << 3));
+}
+
+// Lane a < gd: what row a of U^{-T} amplifies (warp 0), the sum over k of |U^{-T}_ak| |p_k|.
+template <typename T>
+__device__ __forceinline__ float amplification(const T* sLi, const float* sNrm, const int* sExp, int n, int gd) {
+  constexpr int S = kS<T>;
+  const int lane = threadIdx.x & 31;
+  float amp = 0.f;
+  if (lane < gd)
+#pragma unroll 4
+    for (int k = 0; k < S; ++k) {
+      const int q = min(k, n - 1);
+      amp += scaled_abs(sLi[lane * S + k], sExp[q]) * sNrm[q];
+    }
+  return amp;
 }
 
 // 16 bytes of a column in shared memory and their arithmetic: four floats as two packed f32x2
@@ -290,6 +320,68 @@ __device__ __forceinline__ void times_lit(const Blk<T>& c, int jx, int n, const 
   }
 }
 
+// What follows runs only for nearly dependent columns; not inlined, so that it costs the usual
+// path neither registers nor instruction cache.
+
+// Warp 0: the first factor, which covers gd columns, with floored pivots where those are not all of
+// them or a row amplifies more than kMaxHard.  Returns the number of leading columns it covers,
+// and from bit 8 up those of them that amplify rounding by more than kMaxAmp.
+template <typename T>
+__device__ __noinline__ unsigned hard_factor(const T* W, int w, int n, int gd, T* sU, T* sLi, T* sD, T* sRow,
+                                             T* sFl, const float* sNrm, const int* sExp) {
+  constexpr int S = kS<T>;
+  const int lane = threadIdx.x & 31;
+  float amp = amplification(sLi, sNrm, sExp, n, gd);
+  if (gd < n || __any_sync(0xffffffffu, lane > 0 && lane < gd && !(amp <= kMaxHard<T>))) {
+    if (lane < S) sFl[lane] = lane < n ? kFloor<T> * W[lane * w + lane] : T(0);
+    __syncwarp();
+    gd = cholesky<T, true>(W, w, n, sU, sLi, sD, sRow, sFl);
+    amp = amplification(sLi, sNrm, sExp, n, gd);
+    const unsigned bad = __ballot_sync(0xffffffffu, lane > 0 && lane < gd && !(amp <= kMaxHard<T>));
+    if (bad) gd = min(gd, __ffs(bad) - 1);
+  }
+  return (unsigned)gd | __ballot_sync(0xffffffffu, lane > 0 && lane < gd && amp > kMaxAmp) << 8;
+}
+
+// Columns jx .. jx+n-1 <- T with T U = those columns (U upper triangular, element (a, c) at a * S + c;
+// 1 / U_cc at sLi[c * S + c]), by substitution: a thread per row.
+template <typename T>
+__device__ __noinline__ void solve_u(T* P, int rs, int rpc, int n, const T* sU, const T* sLi) {
+  constexpr int S = kS<T>;
+  for (int r = threadIdx.x; r < rpc; r += kNT) {
+    T v[S];
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      T x = k < n ? P[k * rs + r] : T(0);
+#pragma unroll
+      for (int a = 0; a < k; ++a) x -= v[a] * sU[a * S + k];
+      v[k] = x * sLi[k * S + k];
+      if (k < n) P[k * rs + r] = v[k];
+    }
+  }
+}
+
+// The second factor ends before the sub-block (what is left of a column lies in the span of those
+// before it, to rounding): columns n2 .. n1-1 back to T U, from which the column recurrence goes
+// on, and minus their rows of R so far, U2 U, into Y.
+template <typename T>
+__device__ __noinline__ void give_back(T* P, int rs, int rpc, int n1, int n2, const T* sU, const T* sU2, T* Y) {
+  constexpr int S = kS<T>, SY = kSY<T>;
+  for (int r = threadIdx.x; r < rpc; r += kNT)
+    for (int a = n1 - 1; a >= n2; --a) {
+      T x = T(0);
+      for (int k = 0; k <= a; ++k) x += P[k * rs + r] * sU[k * S + a];
+      P[a * rs + r] = x;
+    }
+  for (int e = threadIdx.x; e < (n1 - n2) * S; e += kNT) {
+    const int a = n2 + e / S, i = e % S;
+    T x = T(0);
+    if (i < n2)
+      for (int k = i; k <= a; ++k) x -= sU2[i * S + k] * sU[k * S + a];
+    Y[a * SY + i] = x;
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t ldq,
                                                        T* __restrict__ R, int64_t ldr, int64_t M,
@@ -303,10 +395,11 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ __align__(16) T sU[S * S], sLi[S * S], sU2[S * S];
   __shared__ __align__(16) T sRow[16 * S], sD[S];
+  __shared__ T sFl[S];
   __shared__ float sNrm[S];
   __shared__ int sExp[S];
   __shared__ int sGood;
-  __shared__ unsigned sFail;
+  __shared__ unsigned sFail, sHard;
   const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
   // the slices stay inside the panel's buffers and the sums inside theirs (the same for every
@@ -324,7 +417,7 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
   c.red = c.W + S * bk + bk;
   T* thr = c.red + kNT;  // [bk]
   c.x = Xch{part, fin, ecap, 0u, status, wait_limit};
-  const unsigned tags = 4u * (unsigned)bk + 8u;
+  const unsigned tags = 5u * (unsigned)bk + 8u;
   if (tid < 16 * S) sRow[tid] = T(0);
   if (!exchange_begin(c.x, epoch, tags)) return;
   const unsigned first = c.x.tag;
@@ -349,15 +442,18 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
   const bool icgs = tau2 > 0.0;
   bool ok = true, broke = false;
   int j = 0, w = bk, n = 0, good = 0;
-  unsigned fail = 0u;
+  unsigned fail = 0u, hard = 0u;  // columns that fail the ICGS test, that amplify rounding
   bool second = false;  // the sub-block's second projection (one copy of the code for both)
   while (j < bk) {
     if (!second) {
       w = bk - j;
       n = min(S, w);
     }
-    const int nx = second ? good : n, wx = second ? j + good : w;
-    gram(c, j, nx, second ? 0 : j, wx);
+    // the second projection's products: with the computed columns (off of them; none without the
+    // ICGS test), the sub-block and, if it amplifies rounding, the columns behind it
+    const int off = icgs ? j : 0;
+    const int nx = second ? good : n, wx = second ? off + (hard ? w : good) : w;
+    gram(c, j, nx, second ? j - off : j, wx);
     int E = nx * wx;
     if (j == 0 && icgs && !second) {
       // the squared norms of every column behind the first products
@@ -379,13 +475,13 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
         const int i = idx / good, a = idx - i * good;
         if (a < i) continue;
         T s = T(0);
-        for (int k = lane; k < j; k += 32) s += c.W[i * wx + k] * c.W[a * wx + k];
+        for (int k = lane; k < off; k += 32) s += c.W[i * wx + k] * c.W[a * wx + k];
         s = warp_sum(s);
-        if (lane == 0) c.red[i * S + a] = c.W[i * wx + j + a] - s;
+        if (lane == 0) c.red[i * S + a] = c.W[i * wx + off + a] - s;
       }
       for (int r0 = 0; r0 < rpc; r0 += kNT / 4) {
         const int r = r0 + tid % (kNT / 4), quarter = tid / (kNT / 4);
-        if (r < rpc && j > 0) {
+        if (r < rpc && off > 0) {
           const T* q = c.P + r;
           T acc[S / 4];
           int z[S / 4];
@@ -395,7 +491,7 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
             z[i] = min(4 * i + quarter, good - 1) * wx;
           }
 #pragma unroll 4
-          for (int a = 0; a < j; ++a) {
+          for (int a = 0; a < off; ++a) {
             const T x = q[(size_t)a * rs];
 #pragma unroll
             for (int i = 0; i < S / 4; ++i) acc[i] += x * c.W[z[i] + a];
@@ -434,19 +530,25 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
           sExp[lane] = h;
         }
         __syncwarp();
-        float amp = 0.f;
-        if (lane < gd)
-#pragma unroll 4
-          for (int k = 0; k < S; ++k) {
-            const int q = min(k, n - 1);
-            amp += scaled_abs(sLi[lane * S + k], sExp[q]) * sNrm[q];
-          }
-        const unsigned bad = __ballot_sync(0xffffffffu, lane > 0 && lane < gd && !(amp <= kMaxAmp));
-        if (bad) gd = min(gd, __ffs(bad) - 1);
+        const float amp = amplification(sLi, sNrm, sExp, n, gd);
+        unsigned big = 0u;
+        if (gd < n || __any_sync(0xffffffffu, lane > 0 && lane < gd && !(amp <= kMaxAmp))) {
+          const unsigned r = hard_factor(c.W, w, n, gd, sU, sLi, sD, sRow, sFl, sNrm, sExp);
+          gd = r & 0xff;
+          big = r >> 8;
+        }
         // the ICGS test, from the panel's second column on
         const bool test = icgs && lane < gd && j + lane > 0;
         const unsigned f = __ballot_sync(0xffffffffu, test && sD[test ? lane : 0] < thr[test ? j + lane : 0]);
-        if (lane == 0) sFail = f;
+        if (lane == 0) {
+          sFail = f;
+          sHard = big;
+        }
+      } else {
+        // the pivot of a column of which the second projection takes most has lost its digits
+        const bool ok2 = lane >= gd || sD[lane] >= T(0.25) * c.W[lane * wx + off + lane];
+        const unsigned lost = ~__ballot_sync(0xffffffffu, ok2);
+        if (lost) gd = __ffs(lost) - 1;
       }
     }
     if (tid == 0) sGood = gd;
@@ -454,18 +556,38 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
     if (!second) {
       good = sGood;
       fail = sFail;
-    } else if (sGood < good) {
-      if (g == 0 && tid == 0) set_status(status, CQR_EBREAKDOWN, col0 + j + sGood);
-      broke = true;
-      break;
+      hard = sHard;
+    }
+    const int behind = good;  // the first column behind the sub-block
+    if (second) {
+      // R[0:j, S] += Z1 U by the CTAs that own the columns
+      for (int a = 0; a < good; ++a)
+        if ((j + a) % G == g)
+          for (int i = tid; i < off; i += kNT) {
+            T s = T(0);
+            for (int k = 0; k <= a; ++k) s += c.W[k * wx + i] * sU[k * S + a];
+            R[i + (int64_t)(j + a) * ldr] += s;
+          }
+      if (sGood < good) {
+        give_back<T>(c.P + (size_t)j * rs, rs, rpc, good, sGood, sU, sU2, c.Y);
+        good = sGood;
+        second = good > 0;
+        __syncthreads();
+      }
     }
     if (good > 0) {
       // minus the rows j .. j+good-1 of R, columns j+good .., by columns in Y: four threads
       // (of four warps) per column, S / 4 rows each
-      {
+      if (second || !hard) {
         constexpr int H = S / 4;
         const int quarter = tid / (kNT / 4);
-        for (int a0 = good; a0 < w; a0 += kNT / 4) {
+        // right-hand sides: the products with P_S or, if the first factor amplifies rounding, with T;
+        // else, in the second projection, the rows solved with the first factor (signs: Y's)
+        const bool y = second && !hard;
+        const T* src = y ? c.Y : c.W + (second ? off : 0);
+        const int ss = y ? 1 : wx, sa = y ? SY : 1;
+        const T sg = y ? T(1) : T(-1);
+        for (int a0 = behind; a0 < w; a0 += kNT / 4) {
           const int a = a0 + tid % (kNT / 4);
           T q[H];
 #pragma unroll
@@ -477,7 +599,7 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
 #pragma unroll
               for (int i = 0; i < H; ++i) {
                 const int k = m * H + i;
-                x[i] = k < good ? (second ? c.Y[a * SY + k] : -c.W[k * w + a]) : T(0);
+                x[i] = k < good ? src[k * ss + a * sa] : T(0);
               }
 #pragma unroll
               for (int i = 0; i < H; ++i) {
@@ -490,25 +612,21 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
           if (a < w)
 #pragma unroll
             for (int i = 0; i < H; ++i)
-              c.Y[a * SY + quarter * H + i] = quarter * H + i < good ? q[i] : T(0);
+              c.Y[a * SY + quarter * H + i] = quarter * H + i < good ? sg * q[i] : T(0);
         }
       }
-      times_lit(c, j, good, sLi);  // T = P_S U^{-1}; then Q_S = T U2^{-1}
+      // T = P_S U^{-1}; then Q_S = T U2^{-1}
+      if (hard && !second)
+        solve_u<T>(c.P + (size_t)j * rs, rs, rpc, good, sU, sLi);
+      else
+        times_lit(c, j, good, sLi);
       __syncthreads();
-      if (fail && !second) {
+      if ((fail | hard) && !second) {
         second = true;
         continue;
       }
       if (second) {
-        // R[0:j, S] += Z1 U by the CTAs that own the columns, U <- U2 U
-        for (int a = 0; a < good; ++a)
-          if ((j + a) % G == g)
-            for (int i = tid; i < j; i += kNT) {
-              T s = T(0);
-              for (int k = 0; k <= a; ++k) s += c.W[k * wx + i] * sU[k * S + a];
-              R[i + (int64_t)(j + a) * ldr] += s;
-            }
-        __syncthreads();
+        // U <- U2 U
         if (tid < S * S) {
           const int i = tid / S, a = tid % S;
           T s = T(0);
@@ -518,7 +636,14 @@ __global__ void __launch_bounds__(kNT, 1) k_panel_blk(T* __restrict__ Q, int64_t
         }
         __syncthreads();
         if (tid < S * S) sU[tid] = c.red[tid];
-        if (g == 0 && tid == 0) atomicAdd(status + ST_REORTH, __popc(fail));
+        if (g == 0 && tid == 0 && icgs) {
+          int count = __popc(fail & ((1u << good) - 1u));
+          if (hard) {  // by R's diagonal, since the first pivots miss what a raised one takes
+            count = 0;
+            for (int a = 0; a < good; ++a) count += j + a > 0 && c.red[a * S + a] * c.red[a * S + a] < thr[j + a];
+          }
+          if (count) atomicAdd(status + ST_REORTH, count);
+        }
         __syncthreads();
         second = false;
       }

@@ -48,10 +48,12 @@ __device__ __forceinline__ bool fine_pivot(double d) {
 // their 4 x 4 diagonal block for itself and solves its own column, the solved rows go round, are
 // taken off the rows behind, and those move up by four registers (one rolled loop: straight-line
 // code that runs once per sub-block waits for its instructions).  U into sU[k * S + a] (k <= a),
-// U^{-T} into sLi[k * S + c] (zero for c > k), the pivots into sD; sRow: [2][2 S][4].  Returns
-// the number of leading columns with a fine pivot.
-template <typename T>
-__device__ __forceinline__ int cholesky(const T* B, int ld, int n, T* sU, T* sLi, T* sD, T* sRow) {
+// U^{-T} into sLi[k * S + c] (zero for c > k), the pivots into sD; sRow: [2][2 S][4].  FLOOR: the
+// pivot of column k is fl[k] where it is less (fl[S], zero from n).  Returns the number of leading
+// columns with a fine pivot.
+template <typename T, bool FLOOR = false>
+__device__ __forceinline__ int cholesky(const T* B, int ld, int n, T* sU, T* sLi, T* sD, T* sRow,
+                                        const T* fl = nullptr) {
   constexpr int S = kS<T>;
   const int lane = threadIdx.x & 31;
   T* raw = sRow;              // rows as they stand, [column][4]
@@ -75,6 +77,7 @@ __device__ __forceinline__ int cholesky(const T* B, int ld, int n, T* sU, T* sLi
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       d[q] = m[q][q];
+      if constexpr (FLOOR) d[q] = d[q] < fl[k + q] ? fl[k + q] : d[q];
       // rows behind a bad pivot hold rubbish and are not used
       good = k + q < good && !fine_pivot(d[q]) ? k + q : good;
       iv[q] = inv_root(d[q]);
@@ -88,6 +91,8 @@ __device__ __forceinline__ int cholesky(const T* B, int ld, int n, T* sU, T* sLi
 #pragma unroll
       for (int i = 0; i < q; ++i) x -= m[i][q] * u[i];
       u[q] = x * iv[q];
+      if constexpr (FLOOR)
+        if (lane == k + q) u[q] = d[q] * iv[q];
     }
     if (lane < S)
 #pragma unroll
