@@ -1447,7 +1447,7 @@ __global__ void __launch_bounds__(256) k_ls_cg(const T* __restrict__ Q, int64_t 
     if (!grid_sync(bar, G, target, status, 34)) return;
   }
   for (int64_t j = (int64_t)g * blockDim.x + tid; j < n; j += (int64_t)G * blockDim.x)
-    x[j] = (T)(c > 0 ? __ldcg(w + j) : __ldcg(z + j));
+    x[j] = c > 0 && !isfinite(rr) ? nan_value<T>() : (T)(c > 0 ? __ldcg(w + j) : __ldcg(z + j));
 }
 
 template <typename T>

@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
     p[j] = 0.f;
   }
   __syncthreads();
-  bool ok = true;
+  bool ok = true, finite = true;
   double zz = 0.0, prev = 0.0;
   for (int o = 0; o < kMaxOuter; ++o) {
     // W <- r = z - w + Q_2^T Q_2 w in FP64
@@ -318,6 +318,8 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
     }
     const double rr64 = block_sum(loc, bs);
     if (o == 0) zz = rr64;
+    finite = isfinite(rr64);  // a right-hand side or rows of Q_2 that are not: no x (NaN)
+    if (!finite) break;
     if (!(rr64 > Ends<T>::kOuter * zz) || (o > 0 && !(rr64 < 0.25 * prev))) break;
     prev = rr64;
     const double rn = sqrt(rr64), irn = 1.0 / rn;
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
   }
   exchange_end(epoch, first, kTags);
   if (ok && g == 0)
-    for (int j = tid; j < n; j += kNT) x[j] = (T)w[j];
+    for (int j = tid; j < n; j += kNT) x[j] = finite ? (T)w[j] : nan_value<T>();
 }
 
 }  // namespace
