@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
   }
   __syncthreads();
   bool ok = true, finite = true;
-  double zz = 0.0, prev = 0.0;
+  double zz = 0.0, prev = 0.0, rn = 0.0;
   for (int o = 0; o < kMaxOuter; ++o) {
     // W <- r = z - w + Q_2^T Q_2 w in FP64
     if (o > 0) {
@@ -320,9 +320,14 @@ __global__ void __launch_bounds__(kNT, 1) k_ls_refine(const T* __restrict__ Q, i
     if (o == 0) zz = rr64;
     finite = isfinite(rr64);  // a right-hand side or rows of Q_2 that are not: no x (NaN)
     if (!finite) break;
+    if (o > 0 && rr64 > prev) {  // the correction made it worse: without it
+      for (int j = tid; j < n; j += kNT) w[j] = fma(-rn, (double)d[j], w[j]);
+      break;
+    }
     if (!(rr64 > Ends<T>::kOuter * zz) || (o > 0 && !(rr64 < 0.25 * prev))) break;
     prev = rr64;
-    const double rn = sqrt(rr64), irn = 1.0 / rn;
+    rn = sqrt(rr64);
+    const double irn = 1.0 / rn;
     for (int j = tid; j < n; j += kNT) {
       const float rj = (float)(W[j] * irn);
       r[j] = rj;

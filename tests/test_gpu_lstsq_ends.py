@@ -1,5 +1,7 @@
 """How the tall solve ends (cqr_lstsq.cu, and the conjugate gradients for long vectors): what is not
-finite comes out as NaN and not as a finite x."""
+finite comes out as NaN and not as a finite x, and a correction that makes the residual larger is not
+kept."""
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -65,4 +67,26 @@ def test_a_checksum_row_that_is_not_finite(dtype):
     q.solve_ls(y, x)
     torch.cuda.synchronize()
     assert not bool(torch.isfinite(x).any())
+    q.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("scale", [1.3, 2.0, 3.0])
+def test_a_correction_that_makes_the_residual_larger_is_not_kept(dtype, scale):
+    # checksum rows times `scale`: I - Q_2^T Q_2 is indefinite and conjugate gradients break down
+    q, A, y, x = handle(1003, 96, 2, dtype)
+    Q, R = q.factors()
+    g = q.geo
+    Q2 = Q[g["m_pad"]: g["M"], :96]
+    Q2 *= scale
+    q.solve_ls(y, x)
+    torch.cuda.synchronize()
+    z = Q[:1003, :96].double().t() @ y.double()
+    w = torch.triu(R[:96, :96]).double() @ x.double()
+    Q2 = Q2.double()
+    r = z - (w - Q2.t() @ (Q2 @ w))
+    # w = 0 leaves |z|; x in the storage precision through R (condition number below 2)
+    u = np.finfo(np.float64 if dtype == "f64" else np.float32).eps
+    lim = float(torch.linalg.norm(z)) + 96 * 4 * u * float(torch.linalg.norm(w)) * (1 + scale ** 2)
+    assert float(torch.linalg.norm(r)) <= lim
     q.close()
