@@ -269,10 +269,11 @@ cqr_status coded_qr_stats(cqr_handle h, int64_t* out);
  * none), clearing it. */
 cqr_status coded_qr_sync_status(cqr_handle h);
 
-/* Bound of the waits between the CTAs of one panel factorisation (instrumentation, no
+/* Bound of the waits between the CTAs of one panel factorisation or of one tall solve (instrumentation, no
  * counterpart in the paper; the paper assumes fail-stop nodes and an external failure
- * detector).  Every such wait -- the partial-vector exchange of the cluster panel, the
- * grid barrier of the cooperative panel -- gives up after `cycles` SM clock cycles
+ * detector).  Every such wait -- the sums of the sub-block panel and of the solve by
+ * refinement, the partial-vector exchange of the cluster panel, the grid barrier of the
+ * cooperative panel -- gives up after `cycles` SM clock cycles
  * (0 restores the default, about one second): the CTA records CQR_ETIMEOUT in the device
  * status word, every CTA of the launch leaves at its next wait, and coded_qr_sync_status
  * returns CQR_ETIMEOUT.  The factors computed after that are not meaningful; a new encode

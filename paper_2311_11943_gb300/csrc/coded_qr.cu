@@ -860,7 +860,8 @@ cudaError_t ls_middle(cqr_handle h, int k, const T* y, int64_t ldy, const T* u, 
   const Geo& g = h->g;
   bool taken = false;
   cudaError_t e = launch_ls_refine<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, k, y, ldy, u, ldu,
-                                      w, ldw, h->B.cg, h->B.lsx, h->B.status, h->num_sms, h->st, &taken);
+                                      w, ldw, h->B.cg, h->B.lsx, h->B.status, h->num_sms, h->st, h->wait_limit,
+                                      &taken);
   if (taken || e != cudaSuccess) return e;
   for (int j = 0; j < k && e == cudaSuccess; ++j)
     e = launch_ls_cg<T>(ptr<T>(h->B.Q), g.ldq, g.m, g.m_pad, g.c, g.n, y ? y + j * ldy : nullptr,

@@ -199,7 +199,7 @@ template <typename T>
 cudaError_t launch_ls_refine(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, int64_t c, int64_t n,
                              int k, const T* y, int64_t ldy, const T* u, int64_t ldu, T* x,
                              int64_t ldx, double* z, void* xws, int* status, int num_sms,
-                             cudaStream_t st, bool* taken);
+                             cudaStream_t st, long long wait_limit, bool* taken);
 
 // ---------------------------------------------------------------- adjoint building blocks
 // C (M x N) = alpha op(A) op(B) + beta C (op = transpose when ta / tb); beta == 0 ignores C.

@@ -388,7 +388,7 @@ template <typename T>
 cudaError_t launch_ls_refine(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, int64_t c, int64_t n,
                              int k, const T* y, int64_t ldy, const T* u, int64_t ldu, T* x,
                              int64_t ldx, double* z, void* xws, int* status, int num_sms,
-                             cudaStream_t st, bool* taken) {
+                             cudaStream_t st, long long wait_limit, bool* taken) {
   LsPlan p{};
   *taken = plan_ls(c, n, sizeof(T), num_sms, &p);
   if (!*taken) return cudaSuccess;
@@ -397,7 +397,7 @@ cudaError_t launch_ls_refine(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, 
   if (e != cudaSuccess) return e;
   int ecap = (int)(2 * n);
   unsigned char* xw = static_cast<unsigned char*>(xws);
-  long long wl = kWaitLimitCycles;
+  long long wl = wait_limit > 0 ? wait_limit : kWaitLimitCycles;
   const double* zc = z;
   // one CTA per SM, and (G + 1) ecap words per right-hand side of the (SMs + 1) ecap there are
   const int at_once = std::max(1, std::min({kMaxRhs, num_sms / p.G, (num_sms + 1) / (p.G + 1)}));
@@ -418,11 +418,12 @@ cudaError_t launch_ls_refine(const T* Q, int64_t ldq, int64_t m, int64_t m_pad, 
 
 template cudaError_t launch_ls_refine<float>(const float*, int64_t, int64_t, int64_t, int64_t, int64_t,
                                              int, const float*, int64_t, const float*, int64_t, float*,
-                                             int64_t, double*, void*, int*, int, cudaStream_t, bool*);
+                                             int64_t, double*, void*, int*, int, cudaStream_t, long long,
+                                             bool*);
 template cudaError_t launch_ls_refine<double>(const double*, int64_t, int64_t, int64_t, int64_t,
                                               int64_t, int, const double*, int64_t, const double*,
                                               int64_t, double*, int64_t, double*, void*, int*, int,
-                                              cudaStream_t, bool*);
+                                              cudaStream_t, long long, bool*);
 
 cudaError_t bounds_take_lstsq(int* code, int* site) { return bounds_take_here(code, site); }
 
