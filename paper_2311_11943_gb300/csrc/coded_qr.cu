@@ -191,6 +191,7 @@ struct cqr_handle_s {
   size_t esz = 8;
   double tau = 0.7071067811865476;
   TcGemm* tc = nullptr;
+  bool tc_stale = true;  // columns written since the last update (encode, recovery)
   F64Gemm* f64 = nullptr;
   PanelPlan plan{};
   int plan_bk = -1;
@@ -536,7 +537,7 @@ cqr_status tc_update_cols(cqr_handle h, int64_t kb, int bk, int64_t j0, int64_t 
   }
   {
     ProfScope ps(h, K_SPLITK_REDUCE, 1, st);
-    CK(tc_reduce(h->tc, kb, bk, j0, w, ptr<float>(h->B.R), h->g.ldr, ctx, max_ctas, st));
+    CK(tc_reduce(h->tc, kb, bk, j0, w, ptr<float>(h->B.R), h->g.ldr, buf, ctx, max_ctas, st));
   }
   {
     ProfScope ps(h, K_TC_UPDATE, 1, st);
@@ -798,6 +799,7 @@ cqr_status recover_t(cqr_handle h, int32_t* n_recovered) {
   }
   std::fill(h->mask.begin(), h->mask.end(), 0);
   h->pending = false;
+  h->tc_stale = true;
   h->n_recovered += nrec;
   if (n_recovered) *n_recovered = nrec;
   return CQR_OK;
@@ -990,6 +992,7 @@ cqr_status coded_qr_encode(cqr_handle h, const void* A, int64_t lda) {
   h->postorth_inplace = false;
   h->next_panel = 0;
   h->n_recovered = h->panels_run = h->n_injected = 0;
+  h->tc_stale = true;
   h->state = ST_ENCODED;
   return CQR_OK;
 }
@@ -999,9 +1002,10 @@ cqr_status coded_qr_factor(cqr_handle h, int32_t t0, int32_t t1) {
   if (h->state == ST_CREATED || h->pending || h->postorth_inplace) return CQR_ESTATE;
   if (t1 < 0) t1 = h->g.panels;
   if (t0 != h->next_panel || t1 < t0 || t1 > h->g.panels) return CQR_ESTATE;
-  if (h->tc && t0 == 0 && t1 > 0) {
+  if (h->tc && h->tc_stale && t1 > t0) {
     ProfScope ps(h, K_TC_SPLIT, 1);
-    CK(tc_begin(h->tc, h->st));
+    CK(tc_begin(h->tc, t0 & 1, h->st));
+    h->tc_stale = false;
   }
   if (t1 > t0 && h->esz == 4 && lookahead_eligible(h)) {
     cqr_status s = factor_lookahead(h, t0, t1);

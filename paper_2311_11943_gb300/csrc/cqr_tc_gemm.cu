@@ -22,10 +22,12 @@
 // and so recovers about FP32 accuracy.  The halves are FP16, which has TF32's 11 bits in half the
 // bytes and at twice the rate; what FP16 lacks, TF32's exponent range, comes from a power of two
 // per column (exact to apply and to take out): orthonormal columns are multiplied by 2^12,
-// trailing columns by the power that took their norm into [2^9, 2^10) before the first panel
-// (norms only fall as panels are taken out of a column), the columns of a panel by that of their
-// norm when its block pass begins.  Beyond the halves' 22 bits a split is then off by at most
-// 2^-34 of the column's norm per entry, 2^-10 of the FP32 rounding of the column itself.  Measured
+// trailing columns and those of Rbar by the power that takes their largest magnitude into [2^13,
+// 2^14), the columns of a panel by that which takes their norm into [2^9, 2^10) when its block pass
+// begins.  An entry keeps its 22 bits down to 2^-16 of the column's largest, and is off by at most
+// 2^-38 of it below.  The magnitudes of the trailing columns are taken by the update that writes
+// them, so what is left of a column whose large part was taken out keeps its digits, and a
+// column that grows (a panel far from orthogonal) does not overflow.  Measured
 // against 64 bits: R of 8192 x 8192 1.4e-5 -> 7.7e-6, of 16384 x 2048 6.9e-6 -> 3.7e-6 relative to
 // TF32 halves (fewer roundings in the accumulators).  8192 x 8192, p = 16, b = 256, all panels:
 // Rbar 5.0 -> 2.95 ms, block pass 8.1 -> 5.4 ms, update 4.94 -> 4.38 ms, and 3.52 ms
@@ -115,6 +117,16 @@ __device__ __forceinline__ void mma_op(uint32_t tmem_d, uint64_t a, uint64_t b, 
         : "memory");
 }
 
+// The FP16 scale of a column from the bits of its largest magnitude: the power of two that takes it
+// into [2^13, 2^14), 1 for a column that is zero or not finite.
+__device__ __forceinline__ float f16_scale(unsigned m) {
+  const int e = (int)(m >> 23);
+  if (m == 0u || e == 255) return 1.f;
+  return __int_as_float(min(253, 267 - max(e, 1)) << 23);
+}
+// 1 / s of a power of two s within 2^-126 .. 2^126
+__device__ __forceinline__ float pow2_inv(float s) { return __int_as_float((254 << 23) - __float_as_int(s)); }
+
 __device__ __forceinline__ float tf32_hi(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -145,10 +157,12 @@ struct TcJob {
   float* out;         // epi 0: P base; epi 1: C base (already offset to column j0)
   int64_t ldo;        // leading dimension of out
   int64_t split_stride;  // epi 0: elements between split partials
-  // FP16 operands: raw B rows are multiplied by bscale (nullptr: bconst) before the split, the
-  // epilogue of C -= D multiplies D by oconst and, column by column, by oinv (nullptr: 1)
-  const float* bscale;
+  // FP16 operands: raw B rows are multiplied by the scale of bmax (nullptr: bconst) before the
+  // split, the epilogue of C -= D multiplies D by oconst and, column by column, by oinv (nullptr:
+  // 1), and with CT leaves the largest magnitudes of the new columns in cmax
+  const unsigned* bmax;
   const float* oinv;
+  unsigned* cmax;
   float bconst, oconst;
   int* status;
 };
@@ -358,9 +372,9 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
         const int split = t % job.splits;
         const int nk = kblocks(split);
         float sc = job.bconst;  // FP16: the scale of this thread's row of the B tile
-        if (KD == kF16 && job.bscale) {
+        if (KD == kF16 && job.bmax) {
           const int64_t j = (int64_t)(t / job.splits / mu) * NP * BN + tt;
-          sc = j < job.ncols ? job.bscale[j] : 1.f;
+          sc = j < job.ncols ? f16_scale(job.bmax[j]) : 1.f;
         }
         bool ok = true;
         for (int kb = 0; kb < nk; ++kb, ++it) {
@@ -470,6 +484,8 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
         const int64_t row = row0 + lane;
         float inv = 1.f;
         if (job.oinv && col0 + lane < job.ncols) inv = job.oinv[col0 + lane];
+        unsigned big = 0u, seen = ~0u;  // what the column has already: most chunks need no atomic
+        if (col0 + lane < job.ncols) seen = *reinterpret_cast<volatile unsigned*>(job.cmax + col0 + lane);
         float v[32];
         tmem_ld32(tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(buf * BN + c * 32), v);
 #pragma unroll
@@ -492,10 +508,30 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
             tma_store_2d(&maps.c, (int)row0, (int)(job.c_col0 + col0), ring_u + s * kCBytes);
             bulk_commit();
           }
-        } else if (row < job.mrows) {
-          for (int i = 0; i < 32; ++i)
-            if (col0 + i < job.ncols) job.out[row + (col0 + i) * job.ldo] -= v[i];
+          // column `lane` of the chunk again, along its row of the box (no bank conflicts): 32 reads
+          // across the lanes by __reduce_max_sync cost as much as a tenth of the launch
+          const float4* y = reinterpret_cast<const float4*>(ring + s * kCBytes + lane * 128);
+          float m = 0.f;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float4 c4 = y[k ^ (lane & 7)];
+            m = fmaxf(fmaxf(m, fmaxf(fabsf(c4.x), fabsf(c4.y))), fmaxf(fabsf(c4.z), fabsf(c4.w)));
+          }
+          big = __float_as_uint(m);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float c = 0.f;
+            if (row < job.mrows && col0 + i < job.ncols) {
+              float* x = job.out + row + (col0 + i) * job.ldo;
+              c = *x - v[i];
+              *x = c;
+            }
+            const unsigned m = __reduce_max_sync(~0u, __float_as_uint(c) & 0x7fffffffu);
+            if (lane == i) big = m;
+          }
         }
+        if (big > seen) atomicMax(job.cmax + col0 + lane, big);
       }
       tc_fence_before();
       __syncwarp();
@@ -797,8 +833,7 @@ __global__ void __launch_bounds__(256) k_tc_reduce_t(const float* __restrict__ P
 template <typename PT>
 __global__ void k_tc_reduce(const float* __restrict__ P, int splits, int64_t split_stride, int64_t ldp,
                             int bk, int bkp, int64_t w, float* __restrict__ R, int64_t ldr,
-                            int nplanes, PT* __restrict__ Bh, PT* __restrict__ Bl, float oconst,
-                            const float* __restrict__ oinv) {
+                            int nplanes, PT* __restrict__ Bh, PT* __restrict__ Bl) {
   pdl_wait();
   pdl_trigger();
   const int64_t total = (int64_t)bkp * w;
@@ -808,13 +843,109 @@ __global__ void k_tc_reduce(const float* __restrict__ P, int splits, int64_t spl
     float s = 0.f;
     if (i < bk) {
       for (int sp = 0; sp < splits; ++sp) s += P[sp * split_stride + i + j * ldp];
-      s *= oconst;
-      R[i + j * ldr] = oinv ? s * oinv[j] : s;
+      R[i + j * ldr] = s;
     }
     PT h, l;
     hilo(s, nplanes, h, l);
     Bh[idx] = h;
     if (nplanes == 2) Bl[idx] = l;
+  }
+}
+
+// The same for FP16 operands, a warp per column: the partials hold Rbar times `qscale` and the scale
+// of cmax[j], the planes Rbar times the scale of the column's own largest magnitude, whose
+// inverse goes into ri[j]; cnext[j] is cleared for the update behind.
+__global__ void __launch_bounds__(256) k_tc_reduce_f16(const float* __restrict__ P, int splits,
+                                                       int64_t split_stride, int64_t ldp, int bk, int bkp,
+                                                       int64_t w, float* __restrict__ R, int64_t ldr,
+                                                       __half* __restrict__ Bh, __half* __restrict__ Bl,
+                                                       float qinv, const unsigned* __restrict__ cmax,
+                                                       float* __restrict__ ri, unsigned* __restrict__ cnext) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int E = 4;  // entries of a lane in registers
+  const int lane = threadIdx.x & 31;
+  const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (j >= w) return;
+  const float inv = pow2_inv(f16_scale(cmax[j]));
+  const float* p = P + j * ldp;
+  float* r = R + j * ldr;
+  float v[E];
+  unsigned m = 0u;
+  for (int i0 = 0; i0 < bkp; i0 += 32 * E) {
+#pragma unroll
+    for (int u = 0; u < E; ++u) v[u] = 0.f;
+    int sp = 0;
+    for (; sp + 4 <= splits; sp += 4) {  // the loads of four partials in flight, added in their order
+      float x[4][E];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+          const int i = i0 + 32 * u + lane;
+          x[q][u] = i < bk ? p[(sp + q) * split_stride + i] : 0.f;
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < E; ++u) v[u] += x[q][u];
+    }
+    for (; sp < splits; ++sp)
+#pragma unroll
+      for (int u = 0; u < E; ++u) {
+        const int i = i0 + 32 * u + lane;
+        if (i < bk) v[u] += p[sp * split_stride + i];
+      }
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      const int i = i0 + 32 * u + lane;
+      v[u] = v[u] * qinv * inv;
+      if (i < bk) r[i] = v[u];
+      m = max(m, __float_as_uint(v[u]) & 0x7fffffffu);
+    }
+  }
+  m = __reduce_max_sync(~0u, m);
+  const float s = f16_scale(m);
+  if (lane == 0) {
+    ri[j] = pow2_inv(s);
+    cnext[j] = 0u;
+  }
+  for (int i0 = 0; i0 < bkp; i0 += 32 * E) {
+    if (bkp > 32 * E)  // written above by this lane
+#pragma unroll
+      for (int u = 0; u < E; ++u) {
+        const int i = i0 + 32 * u + lane;
+        v[u] = i < bk ? r[i] : 0.f;
+      }
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      const int i = i0 + 32 * u + lane;
+      if (i >= bkp) continue;
+      __half h, l;
+      hilo(v[u] * s, 2, h, l);
+      Bh[i + j * bkp] = h;
+      Bl[i + j * bkp] = l;
+    }
+  }
+}
+
+// Bits of the largest magnitude of every column of C (M rows), one CTA per column (a NaN counts as the
+// largest).
+__global__ void __launch_bounds__(256) k_col_max(const float* __restrict__ C, int64_t ldc, int64_t M,
+                                                 unsigned* __restrict__ cmax) {
+  __shared__ unsigned red[8];
+  pdl_wait();
+  pdl_trigger();
+  const float* c = C + (int64_t)blockIdx.x * ldc;
+  unsigned m = 0u;
+#pragma unroll 4
+  for (int64_t r = threadIdx.x; r < M; r += 256) m = max(m, __float_as_uint(c[r]) & 0x7fffffffu);
+  m = __reduce_max_sync(~0u, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) m = max(m, red[k]);
+    cmax[blockIdx.x] = m;
   }
 }
 
@@ -834,7 +965,10 @@ struct TcGemm {
   void *Ak_hi[2], *Ak_lo[2], *At_hi[2], *At_lo[2], *Bh[2], *Bl[2];
   float* P[2];
   void *Qr_hi, *Qr_lo, *Sh, *Sl;   // block reorthogonalisation operands
-  float *cs, *ci;                  // FP16: scales of the N columns and their inverses
+  // FP16: bits of the columns' largest magnitudes at a panel (by its parity) and the inverse scales
+  // of the Rbar planes' columns; in the block pass, scales of the panel's columns and their inverses
+  unsigned* cm[2];
+  float *ri, *cs, *ci;
   int64_t n, ldrow;
   int num_sms;
   int* status;
@@ -1011,7 +1145,7 @@ size_t tc_workspace_bytes(int mode, int64_t M, int64_t N, int64_t n, int b, int 
     s += 2 * al256((size_t)M * ldrow * pe);      // row-major computed columns hi/lo
     s += 2 * al256((size_t)ldrow * akc * pe);    // S planes
   }
-  if (kind_of(mode) == kF16) s += 2 * al256((size_t)N * 4);  // column scales
+  if (kind_of(mode) == kF16) s += 5 * al256((size_t)N * 4);  // column scales
   return s;
 }
 
@@ -1054,8 +1188,12 @@ TcGemm* tc_create(int mode, int64_t M, int64_t N, int64_t n, int64_t b, float* Q
     t->Sh = take((size_t)t->ldrow * akc * pe);
     t->Sl = take((size_t)t->ldrow * akc * pe);
   }
-  t->cs = t->ci = nullptr;
+  t->cs = t->ci = t->ri = nullptr;
+  t->cm[0] = t->cm[1] = nullptr;
   if (t->kind == kF16) {
+    t->cm[0] = static_cast<unsigned*>(take((size_t)N * 4));
+    t->cm[1] = static_cast<unsigned*>(take((size_t)N * 4));
+    t->ri = static_cast<float*>(take((size_t)N * 4));
     t->cs = static_cast<float*>(take((size_t)N * 4));
     t->ci = static_cast<float*>(take((size_t)N * 4));
   }
@@ -1127,12 +1265,12 @@ int tc_splits(const TcGemm* t, int m1, int n1, int64_t* kchunk, int max_ctas = 0
 }
 }  // namespace
 
-// Scales of all columns, before the first panel: the norms of the trailing columns only fall
-// (up to rounding) as panels are taken out of them, so the scales hold for the whole factor.
-cudaError_t tc_begin(TcGemm* t, cudaStream_t st) {
+// The largest magnitudes of all columns as they are before the panel of parity `buf`; each update leaves
+// those of its columns for the next panel.
+cudaError_t tc_begin(TcGemm* t, int buf, cudaStream_t st) {
   if (t->kind != kF16) return cudaSuccess;
-  return launch_k(k_col_scale, dim3((unsigned)t->N), dim3(256), 0, st, t->pdl && st == t->pdl_st,
-                  (const float*)t->Q, t->ldq, t->M, t->cs, t->ci);
+  return launch_k(k_col_max, dim3((unsigned)t->N), dim3(256), 0, st, t->pdl && st == t->pdl_st,
+                  (const float*)t->Q, t->ldq, t->M, t->cm[buf]);
 }
 
 namespace {
@@ -1178,8 +1316,8 @@ cudaError_t tc_refresh_rect(TcGemm* t, int64_t r0, int64_t nr, int64_t c0, int64
 
 // 2. GEMM1, split-K over the M rows: partials P[s] = Qbar^T Q[:, j0 : j0+w]
 namespace {
-// bscale: FP16 scales of the columns j0.. of Q (nullptr: orthonormal columns)
-cudaError_t gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, const float* bscale, int buf, int ctx,
+// bmax: FP16, the largest magnitudes of the columns j0.. of Q (nullptr: orthonormal columns)
+cudaError_t gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, const unsigned* bmax, int buf, int ctx,
                       int max_ctas, cudaStream_t st) {
   const int three = t->nplanes == 2;
   const int bkp = (int)t->bkp;
@@ -1210,7 +1348,7 @@ cudaError_t gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, const float* bsc
   job.out = t->P[ctx];
   job.ldo = bkp;
   job.split_stride = (int64_t)bkp * w;
-  job.bscale = bscale;
+  job.bmax = bmax;
   job.bconst = q_scale(t);
   job.status = t->status;
   return launch_mode(t, split, maps, job, st, max_ctas);
@@ -1219,12 +1357,12 @@ cudaError_t gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, const float* bsc
 
 cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int ctx, int max_ctas,
                          cudaStream_t st) {
-  return gemm_rbar(t, bk, j0, w, t->kind == kF16 ? t->cs + j0 : nullptr, buf, ctx, max_ctas, st);
+  return gemm_rbar(t, bk, j0, w, t->kind == kF16 ? t->cm[buf] + j0 : nullptr, buf, ctx, max_ctas, st);
 }
 
 // 3. reduce the partials into R[kb.., j0..] and GEMM2's B planes
 cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, float* R, int64_t ldr,
-                      int ctx, int max_ctas, cudaStream_t st) {
+                      int buf, int ctx, int max_ctas, cudaStream_t st) {
   const int bkp = (int)t->bkp;
   const int m1 = (bk + BM - 1) / BM;
   const int n1 = (int)((w + BN - 1) / BN);
@@ -1235,12 +1373,18 @@ cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, floa
   const bool pdl = t->pdl && st == t->pdl_st;
   const float* P = t->P[ctx];
   float* Rd = R + kb + j0 * ldr;
-  return with_plane(t, [&](auto tag) {
+  if (t->kind == kF16)
+    return launch_k(k_tc_reduce_f16, dim3((unsigned)((w + 7) / 8)), dim3(256), 0, st, pdl, P, splits,
+                    (int64_t)bkp * w, (int64_t)bkp, bk, bkp, w, Rd, ldr, pl<__half>(t->Bh[ctx]),
+                    pl<__half>(t->Bl[ctx]), q_inv(t), (const unsigned*)(t->cm[buf] + j0), t->ri + j0,
+                    t->cm[buf ^ 1] + j0);
+  auto go = [&](auto tag) {
     using P_ = decltype(tag);
     return launch_k(k_tc_reduce<P_>, dim3(blocks), dim3(256), 0, st, pdl, P, splits, (int64_t)bkp * w,
                     (int64_t)bkp, bk, bkp, w, Rd, ldr, t->nplanes, pl<P_>(t->Bh[ctx]),
-                    pl<P_>(t->Bl[ctx]), q_inv(t), inv_of(t, j0));
-  });
+                    pl<P_>(t->Bl[ctx]));
+  };
+  return t->kind == kBF16 ? go(__nv_bfloat16{}) : go(float{});
 }
 
 // 4. GEMM2: Q[:, j0 : j0+w] -= Qbar Rbar (M tiles over rows, N tiles over trailing columns)
@@ -1272,8 +1416,9 @@ cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, in
   job.status = t->status;
   job.c_col0 = j0;
   job.oconst = q_inv(t);
-  job.oinv = inv_of(t, j0);
   if (t->kind == kF16) {
+    job.oinv = t->ri + j0;
+    job.cmax = t->cm[buf ^ 1] + j0;
     maps.c = t->tm_q_c;
     return launch_gemm<kF16, false, 2, 2, 2, 1, 1, true>(
         maps, job, max_ctas > 0 ? std::min(max_ctas, t->num_sms) : t->num_sms, st,

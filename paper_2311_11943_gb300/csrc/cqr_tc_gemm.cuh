@@ -19,8 +19,9 @@ void tc_set_status(TcGemm* t, int* status);
 // With `on`, launches on stream st (and only there) use programmatic dependent launch: each kernel waits
 // for its predecessor's completion before touching data, then lets its successor launch.
 void tc_set_pdl_stream(TcGemm* t, bool on, cudaStream_t st);
-// Before panel 0: what the operands need to know of the encoded matrix (FP16: column scales).
-cudaError_t tc_begin(TcGemm* t, cudaStream_t st);
+// Before the panel of parity buf, when the columns are not as its last update left them (encoded, or
+// recovered): what the operands need to know of them (FP16: their largest magnitudes).
+cudaError_t tc_begin(TcGemm* t, int buf, cudaStream_t st);
 // The trailing update of one panel, in four stream-ordered launches:
 //   split the panel into operand planes; Rbar partials = Qbar^T Q[:, j0:j0+w] (split-K);
 //   reduce into R[kb:kb+bk, j0:j0+w] and GEMM2's operand; Q[:, j0:j0+w] -= Qbar Rbar.
@@ -32,7 +33,7 @@ cudaError_t tc_split_panel(TcGemm* t, int64_t kb, int bk, int buf, cudaStream_t 
 cudaError_t tc_gemm_rbar(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int ctx, int max_ctas,
                          cudaStream_t st);
 cudaError_t tc_reduce(TcGemm* t, int64_t kb, int bk, int64_t j0, int64_t w, float* R, int64_t ldr,
-                      int ctx, int max_ctas, cudaStream_t st);
+                      int buf, int ctx, int max_ctas, cudaStream_t st);
 cudaError_t tc_gemm_update(TcGemm* t, int bk, int64_t j0, int64_t w, int buf, int ctx, int max_ctas,
                            cudaStream_t st);
 
