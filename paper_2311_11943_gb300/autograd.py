@@ -30,6 +30,29 @@ def _cm(t, rows=None):
     return out
 
 
+def _workspaces(count, cfg):
+    """Workspaces from the tensor allocator of the current stream: the handles of one call are made
+    and dropped together, and an allocation and a free of 250 MB from the driver cost 0.3 ms each.
+    Of the caller's stream, so that the next call takes the same blocks whatever its side streams."""
+    nbytes = B.coded_qr_workspace_size(cfg) + 256
+    try:
+        return [torch.empty(nbytes, dtype=torch.uint8, device="cuda") for _ in range(count)]
+    except torch.cuda.OutOfMemoryError as e:
+        raise B.CodedQRError(B.CQR_ENOMEM, "coded_qr_create_in") from e
+
+
+def _with_room(verb, *args):
+    """verb(*args); once more with the allocator's unused blocks given back if memory ran out (the
+    library's own scratch comes from the driver)."""
+    try:
+        return verb(*args)
+    except B.CodedQRError as e:
+        if e.status != B.CQR_ENOMEM:
+            raise
+    torch.cuda.empty_cache()
+    return verb(*args)
+
+
 class CodedLstsqFunction(torch.autograd.Function):
     """(Q, R, x) = coded_lstsq(A, y); A (batch, m, n), y (batch, m, k)."""
 
@@ -47,18 +70,16 @@ class CodedLstsqFunction(torch.autograd.Function):
         Q = torch.empty((batch, m, n), dtype=A.dtype, device=A.device)
         R = torch.empty((batch, n, n), dtype=A.dtype, device=A.device)
         X = torch.empty((batch, n, k), dtype=A.dtype, device=A.device)
+        shape = (m, n, opts["p_r"], opts["p_c"], opts["f"], opts["b"])
+        cfg = dict(dtype=dt, mma=mma, nrhs_max=k, seed=opts.get("seed", 1), tau=opts.get("tau", 0.0))
+        spaces = _workspaces(batch, B.make_config(*shape, **cfg))
         for s in streams:
-            s.wait_stream(cur)
+            s.wait_stream(cur)  # after the allocations: their blocks' earlier uses lie on cur
         saved = []
         for i in range(batch):
             s = streams[i % len(streams)]
             with torch.cuda.stream(s):
-                # workspace from the tensor allocator of this stream: the handles of one call
-                # are made and dropped together, and an allocation and a free of 250 MB from the
-                # driver cost 0.3 ms each
-                q = B.CodedQR(m, n, opts["p_r"], opts["p_c"], opts["f"], opts["b"], dtype=dt,
-                              mma=mma, nrhs_max=k, seed=opts.get("seed", 1),
-                              tau=opts.get("tau", 0.0), stream=s, workspace="torch")
+                q = B.CodedQR(*shape, **cfg, stream=s, workspace=spaces.pop())
                 Ac = _cm(A[i])
                 yc = _cm(y[i])
                 q.encode(Ac)
@@ -111,13 +132,13 @@ class CodedLstsqFunction(torch.autograd.Function):
                 if Qbar is not None or Rbar is not None:
                     Qb = _cm(Qbar[i], rows=q.geo["m_pad"]) if Qbar is not None else None
                     Rb = _cm(torch.triu(Rbar[i])) if Rbar is not None else None
-                    q.adjoint_qr(Qo, Qb, Rb, Ab)
+                    _with_room(q.adjoint_qr, Qo, Qb, Rb, Ab)
                     keep += [t_ for t_ in (Qb, Rb) if t_ is not None]
                 if xbar is not None:
                     yb = B.colmajor_empty(m, k, Abar.dtype)
                     yb.zero_()
                     xb = _cm(xbar[i])
-                    q.adjoint_lstsq(Ac, yc, xc, xb, Ab, yb)
+                    _with_room(q.adjoint_lstsq, Ac, yc, xc, xb, Ab, yb)
                     ybar[i].copy_(yb)
                     keep += [yb, xb]
                 Abar[i].copy_(Ab)

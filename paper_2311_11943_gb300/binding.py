@@ -451,8 +451,33 @@ def _ld(t):
     return t.stride(1) if t.shape[1] > 1 else max(t.shape[0], 1)
 
 
+def make_config(m, n, p_r, p_c, f, b, dtype="f64", mma="simt", protect_r=True, gdist=CQR_G_UNIF01,
+                nrhs_max=1, seed=1, tau=0.0, stream=None, reorth_block=False, panel="icgs",
+                in_node=False, post_orth="auto"):
+    """The configuration record of CodedQR's arguments (stream: a torch stream)."""
+    cfg = Config()
+    cfg.m, cfg.n, cfg.p_r, cfg.p_c, cfg.f, cfg.b = m, n, p_r, p_c, f, b
+    cfg.dtype = CQR_F64 if dtype in ("f64", "float64") else CQR_F32
+    cfg.mma = MMA_NAMES[mma]
+    cfg.protect_r = int(bool(protect_r))
+    cfg.gdist = gdist
+    cfg.nrhs_max = nrhs_max
+    cfg.reorth_block = int(bool(reorth_block))
+    cfg.panel = PANEL_NAMES[panel]
+    cfg.in_node = int(bool(in_node))
+    cfg.post_orth = POST_ORTH_NAMES[post_orth]
+    cfg.seed = seed
+    cfg.tau = tau
+    cfg.stream = C.c_void_p(stream.cuda_stream if stream is not None else None)
+    return cfg
+
+
 class CodedQR:
-    """One coded QR problem on the current CUDA device (handle wrapper)."""
+    """One coded QR problem on the current CUDA device (handle wrapper).
+
+    workspace: None (the library allocates), "torch" (from the tensor allocator of the current
+    stream) or a uint8 tensor of coded_qr_workspace_size + 256 bytes, whose earlier uses the
+    handle's stream has waited for; it is held until close, which waits for the handle's work."""
 
     def __init__(self, m, n, p_r, p_c, f, b, dtype="f64", mma="simt", protect_r=True,
                  gdist=CQR_G_UNIF01, nrhs_max=1, seed=1, tau=0.0, stream=None, workspace=None,
@@ -460,26 +485,18 @@ class CodedQR:
         import torch
         self.torch = torch
         self.tdtype = torch.float64 if dtype in ("f64", "float64") else torch.float32
-        cfg = Config()
-        cfg.m, cfg.n, cfg.p_r, cfg.p_c, cfg.f, cfg.b = m, n, p_r, p_c, f, b
-        cfg.dtype = CQR_F64 if self.tdtype == torch.float64 else CQR_F32
-        cfg.mma = MMA_NAMES[mma]
-        cfg.protect_r = int(bool(protect_r))
-        cfg.gdist = gdist
-        cfg.nrhs_max = nrhs_max
-        cfg.reorth_block = int(bool(reorth_block))
-        cfg.panel = PANEL_NAMES[panel]
-        cfg.in_node = int(bool(in_node))
-        cfg.post_orth = POST_ORTH_NAMES[post_orth]
-        cfg.seed = seed
-        cfg.tau = tau
         if stream is None:
             stream = torch.cuda.current_stream()
         self.stream = stream
-        cfg.stream = C.c_void_p(stream.cuda_stream)
+        cfg = make_config(m, n, p_r, p_c, f, b, dtype, mma, protect_r, gdist, nrhs_max, seed, tau,
+                          stream, reorth_block, panel, in_node, post_orth)
         self.cfg = cfg
         self._ws = None
-        if workspace == "torch":
+        if workspace is not None and not isinstance(workspace, str):
+            self._ws = workspace
+            base = (workspace.data_ptr() + 255) // 256 * 256
+            self.h = coded_qr_create_in(cfg, base, workspace.data_ptr() + workspace.numel() - base)
+        elif workspace == "torch":
             nbytes = coded_qr_workspace_size(cfg)
             self._ws = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
             base = (self._ws.data_ptr() + 255) // 256 * 256
@@ -492,6 +509,7 @@ class CodedQR:
         if getattr(self, "h", None):
             coded_qr_destroy(self.h)
             self.h = None
+            self._ws = None
 
     def __del__(self):
         try:
