@@ -875,27 +875,20 @@ __global__ void __launch_bounds__(256) k_tc_reduce_f16(const float* __restrict__
   for (int i0 = 0; i0 < bkp; i0 += 32 * E) {
 #pragma unroll
     for (int u = 0; u < E; ++u) v[u] = 0.f;
-    int sp = 0;
-    for (; sp + 4 <= splits; sp += 4) {  // the loads of four partials in flight, added in their order
-      float x[4][E];
+    for (int sp = 0; sp < splits; sp += 8) {  // the loads of eight partials in flight, added in their order
+      float x[8][E];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < 8; ++q)
 #pragma unroll
         for (int u = 0; u < E; ++u) {
           const int i = i0 + 32 * u + lane;
-          x[q][u] = i < bk ? p[(sp + q) * split_stride + i] : 0.f;
+          x[q][u] = i < bk && sp + q < splits ? p[(sp + q) * split_stride + i] : 0.f;
         }
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < 8; ++q)
 #pragma unroll
         for (int u = 0; u < E; ++u) v[u] += x[q][u];
     }
-    for (; sp < splits; ++sp)
-#pragma unroll
-      for (int u = 0; u < E; ++u) {
-        const int i = i0 + 32 * u + lane;
-        if (i < bk) v[u] += p[sp * split_stride + i];
-      }
 #pragma unroll
     for (int u = 0; u < E; ++u) {
       const int i = i0 + 32 * u + lane;
