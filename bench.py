@@ -1042,8 +1042,11 @@ def run_panels(args):
         Ad = B.colmajor_empty(cfg["m"], cfg["n"], torch.float32)
         Ad.copy_(torch.from_numpy(np.ascontiguousarray(A_np)))
         A64 = torch.from_numpy(A_np).cuda()
-        for panel, reg in (("icgs", "1"), ("icgs", "0"), ("mgs", "0"), ("cgs1", "0"), ("cgs2", "0")):
-            os.environ["CQR_PANEL_REG"] = reg
+        for panel, kernel in (("icgs", "sub-block"), ("icgs", "register"), ("icgs", "shared-memory"),
+                              ("mgs", "sub-block"), ("mgs", "shared-memory"),
+                              ("cgs1", "shared-memory"), ("cgs2", "shared-memory")):
+            os.environ["CQR_PANEL_BLK"] = "1" if kernel == "sub-block" else "0"
+            os.environ["CQR_PANEL_REG"] = "0" if kernel == "shared-memory" else "1"
             q = B.CodedQR(cfg["m"], cfg["n"], cfg["p_r"], cfg["p_c"], cfg["f"], cfg["b"],
                           dtype="f32", mma="3xtf32", seed=cfg["seed"], panel=panel,
                           reorth_block=True)
@@ -1064,9 +1067,10 @@ def run_panels(args):
             q.close()
             pm = prof["panel_icgs"][0] / args.steps
             rows.append({"kappa": kappa, "panel": panel,
-                         "kernel": "register" if (panel == "icgs" and reg == "1") else "shared-memory",
+                         "kernel": kernel,
                          "panel_ms_per_factorisation": pm, "us_per_column": pm * 1e3 / n,
                          "orth_coded_Q": orth, "backward_rel_fro": back, "status": st})
+    os.environ.pop("CQR_PANEL_BLK", None)
     os.environ.pop("CQR_PANEL_REG", None)
     best = min(r["panel_ms_per_factorisation"] for r in rows)
     line = {"metric": "panel factorisation time per C2 factorisation (NEXT f3 comparison)",

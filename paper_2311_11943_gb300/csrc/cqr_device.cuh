@@ -9,8 +9,8 @@
 namespace cqr {
 
 // Device status word layout (int[4]): [0] first error code (CQR_*), [1] reorthogonalisation
-// count, [2] detail of the first error (e.g. the global column of a breakdown), [3] the
-// barrier site that timed out.
+// count, [2] detail of the first error (the global column of a breakdown, the site of a wait that
+// ran out), [3] the site again where the wait was a grid barrier's.
 enum { ST_CODE = 0, ST_REORTH = 1, ST_DETAIL = 2, ST_SITE = 3 };
 
 __device__ __forceinline__ void set_status(int* st, int code, int detail) {

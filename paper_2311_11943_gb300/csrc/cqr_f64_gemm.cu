@@ -9,7 +9,8 @@
 // two numbers is sum over (i, j) of digit products of weight 256^-(i+j); the pairs of equal
 // i + j = g < 7 are summed in one FP32 accumulator, exactly, since 256 products of two 7-bit
 // magnitudes times the at most four pairs that have to be exact stay below 2^24 (the sums of g > 3
-// may round, at weights below 2^-56).  Every 256 of K the seven accumulators are read, converted
+// may round, when all of their digits are near the largest: by a unit of their group, for g = 4
+// 2^-46 of one product of the largest magnitudes and 2^-54 of the sum of 256 of them).  Every 256 of K the seven accumulators are read, converted
 // and added up, exactly, in one 76-bit integer per output (64 bits in units of 2^12 and a 16-bit
 // remainder), which becomes a double once, at the end.  What is lost are the dropped pairs
 // (g >= 7) and the rounding of the operands, each below 2^-53 of a product of the largest

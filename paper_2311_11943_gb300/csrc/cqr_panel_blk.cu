@@ -22,11 +22,13 @@
 // depends on the first factor: T = P_S U^{-1} by substitution (P_S = T U to rounding), the
 // rows of R behind the sub-block from products with T (the second projection's products then
 // run over all columns), and a pivot below kFloor times its column's squared norm is raised to
-// that, which only scales its column of T.  A column whose second norm cannot be had this way either
-// (amplification above kMaxHard) or whose pivot is not positive and finite goes through the column
-// recurrence itself (products, ICGS reorthogonalisation when the test asks for it, normalisation,
-// update), and the next sub-block starts behind it.  Without the ICGS test (MGS) the second
-// projection is within the sub-block.  Every CTA takes the same decisions from the same sums.
+// that, which only scales its column of T.  The sub-block ends before a column with amplification
+// above kMaxHard or a pivot that is not positive and finite, and, in the second factor, before
+// one of whose norm the projection leaves less than half (its pivot has lost its digits; it is given
+// back as T U).  That column goes through the column recurrence itself (products, ICGS
+// reorthogonalisation when the test asks for it, normalisation, update), and the next sub-block
+// starts behind it.  Without the ICGS test (MGS) the second projection is within the
+// sub-block.  Every CTA takes the same decisions from the same sums.
 // Why not the recurrence for every column above kMaxAmp: 4096 x 2048, b = 128, every second column
 // within 1e-3 of the one before, 24.5 ms that way (8.4 ms by the column-by-column kernels), 4.8 ms
 // so; every seventh column 7.7 (5.8), 4.8 ms.

@@ -8,8 +8,9 @@ namespace cqr {
 // Columns per sub-block: 16 in FP32; 8 in FP64, whose S x S factor would not stay in registers.
 template <typename T>
 constexpr int kS = sizeof(T) == 4 ? 16 : 8;
-// A sub-block is cut where a row of U^{-T} amplifies rounding by more than this (the sum over k of
-// |U^{-T}_ak| |p_k|, 1 for orthogonal columns).
+// Rows of U^{-T} that amplify rounding by more than this (the sum over k of |U^{-T}_ak| |p_k|, 1 for
+// orthogonal columns) are not used as they are: a batch cuts the sub-block there, a single
+// problem's panel projects it a second time.
 constexpr float kMaxAmp = 4.0f;
 
 // 1 / sqrt(d) for positive finite d from an FP32 estimate y of relative error e / 2, where

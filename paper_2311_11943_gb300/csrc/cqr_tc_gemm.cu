@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(Warps<KD, SB>::kThreads, 1) k_tc_gemm(const __
 #pragma unroll 1
       for (int u = 0; u < 2; ++u) {
         const int g = 2 * tl + u, s = g % kCSlots, c = half + 2 * u;
-        if (lane == 0) bulk_wait_read();  // the slot of chunk g + 2 was stored from two chunks ago
+        if (lane == 0) bulk_wait_read();  // the slot of chunk g + 2 was stored from by chunk g - 1
         __syncwarp();
         cload(g + 2);
         int64_t row0 = 0, col0 = 0;
