@@ -30,9 +30,9 @@
 // column that grows (a panel far from orthogonal) does not overflow.  Measured
 // against 64 bits: R of 8192 x 8192 1.4e-5 -> 7.7e-6, of 16384 x 2048 6.9e-6 -> 3.7e-6 relative to
 // TF32 halves (fewer roundings in the accumulators).  8192 x 8192, p = 16, b = 256, all panels:
-// Rbar 5.0 -> 2.95 ms, block pass 8.1 -> 5.4 ms, update 4.94 -> 4.38 ms, and 3.52 ms
-// with C through shared memory (CT below; one pass over the trailing columns is 1.6 ms at the copy
-// rate).
+// Rbar 5.0 -> 2.95 ms, block pass 8.1 -> 5.4 ms, update 4.94 -> 4.38 ms, 3.52 ms with C
+// through shared memory (CT below; one pass over the trailing columns is 1.6 ms at the copy
+// rate) and 3.69 ms with the columns' magnitudes.
 // The small operands (panel and Rbar) are split into hi/lo planes in global memory by helper
 // kernels.
 // Every mbarrier wait is bounded: on expiry the kernel records CQR_ETIMEOUT, stops issuing,
