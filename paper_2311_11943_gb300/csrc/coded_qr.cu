@@ -855,7 +855,7 @@ cqr_status post_orth_y(cqr_handle h, const T* y, int64_t ldy, int32_t nrhs, T* y
 
 // ------------------------------------------------------------------------------- solve
 // w = (I - Q_2^T Q_2)^{-1} Q_1^T y (or ... u), k right-hand sides: by iterative refinement where its vectors
-// fit shared memory (n up to about 7000), else by conjugate gradients in FP64.
+// fit shared memory (n up to about 7900), else by conjugate gradients in FP64.
 template <typename T>
 cudaError_t ls_middle(cqr_handle h, int k, const T* y, int64_t ldy, const T* u, int64_t ldu, T* w,
                       int64_t ldw) {
